@@ -180,7 +180,7 @@ dwf_status dwf_create(dwf_t* handle, const int dims[4], int Ls, double M5, doubl
   if (st == DWF_OK) st = build_matrices(h);
   Layout* lay = nullptr;
   if (st == DWF_OK) st = get_layout(h, dims, &lay);
-  if (st == DWF_OK) st = ensure_reduction(h, lay->g.Vp / 32 * 2 + 64, lay->g.nblocks + 64);
+  if (st == DWF_OK) st = ensure_reduction(h, lay->g.Vp + 64, lay->g.nblocks + 64);
   if (st != DWF_OK) {
     std::string msg = dwf_last_error();
     dwf_destroy(h);

@@ -56,7 +56,7 @@ struct Group {
   double* sc = nullptr;        // [8][nseg]: rho, alpha, beta, pap, stop2, rr64, bb, tmp
   int* fl = nullptr;           // [4][nseg]: conv, stop, iter, skip (RU selection)
   unsigned* counter = nullptr; // [nseg]
-  double* partial = nullptr;   // [ntiles]
+  double* partial = nullptr;   // [Vp]
   int grid = 0;                // autotuned persistent grid of the stage launches
   int sgrid = 0, sgather = -1;  // persistent CG-step launch: grid, link staging (tuned;
                                 // gather -1: one launch per stage instead)
@@ -407,7 +407,7 @@ void g_step_args(const Group& G, int nsteps, unsigned long long wait_ns, BatchSt
     x->err = G.err;
     x->wait_ns = wait_ns;
     x->grid = 0;
-    finish_stage_args(*x, G.Ls);
+    finish_stage_args(*x, G.Ls, x == &ad || x == &bd);
   }
   b.A = a;
   b.B = bb;
@@ -576,6 +576,7 @@ dwf_status build_group(Batch& B, Group& G, const dwf_problem* pr) {
       S.dc = P.c;
       S.k64 = make_coef5<double>(la, lb, P.mf, P.b, P.c, 1.0, Ls);
       S.k32 = make_coef5<float>(la, lb, P.mf, P.b, P.c, 1.0, Ls);
+      S.post5 = make_post5(la, lb, P.mf, P.b, P.c, 1.0, Ls);
       S.Vh = (int)P.Vh;
       S.first_tile = (int)P.first_tile;
       S.ntiles = (int)P.ntiles;
@@ -612,7 +613,8 @@ dwf_status build_group(Batch& B, Group& G, const dwf_problem* pr) {
   DWF_TRY(G.alloc(&G.sc, SC_N * G.nseg * sizeof(double)));
   DWF_TRY(G.alloc(&G.fl, FL_N * G.nseg * sizeof(int)));
   DWF_TRY(G.alloc(&G.counter, G.nseg * sizeof(unsigned)));
-  DWF_TRY(G.alloc(&G.partial, (size_t)G.ntiles * sizeof(double)));
+  // one partial per CTA: at the finest one site per CTA (FP64 stages)
+  DWF_TRY(G.alloc(&G.partial, (size_t)G.Vp * sizeof(double)));
   DWF_TRY(G.alloc(&G.bar, sizeof(unsigned)));
   DWF_TRY(G.alloc(&G.err, sizeof(int)));
   DWF_CUDA(cudaMemsetAsync(G.err, 0, sizeof(int), st));

@@ -6,6 +6,7 @@
 #include <type_traits>
 
 #include "dwf_internal.h"
+#include "stage64.cuh"
 #include "vec_tile.cuh"
 
 namespace dwf {
@@ -31,11 +32,12 @@ __global__ void __launch_bounds__(32 * LS) vec_kernel(const VecArgs a) {
 template <int P, int LS>
 static cudaError_t vec_launch(const VecArgs& a, cudaStream_t st) {
   using A = typename Prec<P>::acc;
-  const size_t sm = a.do_u ? (size_t)LS * 24 * 32 * sizeof(A) : 0;
+  const int w = P == P64 ? 1 << stage64_shape(a.Vp, LS, sm_count(), 1).lst : 32;
+  const size_t sm = a.do_u ? (size_t)LS * 24 * w * sizeof(A) : 0;
   static std::atomic<uint64_t> attr{0};
   cudaError_t e = set_smem_once(vec_kernel<P, LS>, attr, (int)(LS * 24 * 32 * sizeof(A)));
   if (e != cudaSuccess) return e;
-  vec_kernel<P, LS><<<dim3((unsigned)(a.Vp / 32)), dim3(32, LS), sm, st>>>(a);
+  vec_kernel<P, LS><<<dim3((unsigned)(a.Vp / w)), dim3(w, LS), sm, st>>>(a);
   return cudaGetLastError();
 }
 

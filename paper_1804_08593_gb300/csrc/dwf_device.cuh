@@ -445,7 +445,6 @@ __device__ void grid_reduce(const RedArgs& r, T (&v)[NV], double* scratch) {
   grid_reduce_seg<NV, T>(r, v, scratch, blockIdx.x, seg, (long)seg * r.cps, r.cps);
 }
 
-// Per-problem description of a batched (concatenated) site space: problem = segment.
 // Fifth-dimension coefficients of a stage in one arithmetic type, computed on the host so
 // that FP32 kernels run no FP64 instructions (GB300's FP64 pipe is narrow):
 // M5op = la + lb K with walls -mf, D+ = db + dc K, and for the recurrence post r = lb/la,
@@ -465,11 +464,29 @@ inline Coef5<A> make_coef5(double la, double lb, double mf, double db, double dc
           A(pre)};
 }
 
+// FP64 recurrence post f D+ M5op^-1 (or f M5op^-dag D+^dag) with its constants folded:
+// pb = f db / la, pc = f dc / la, the wall pcw = -mf pc, cor[t] = kappa (-r)^t.
+struct Post5 {
+  double pb, pc, pcw, cor[16];
+};
+inline Post5 make_post5(double la, double lb, double mf, double db, double dc, double f, int Ls) {
+  const Coef5<double> c = make_coef5<double>(la, lb, mf, db, dc, 1.0, Ls);
+  Post5 p{};
+  p.pb = f * db * c.inva;
+  p.pc = f * dc * c.inva;
+  p.pcw = -mf * p.pc;
+  double g = c.kappa;
+  for (int t = 0; t < Ls && t < 16; t++, g *= -c.r) p.cor[t] = g;
+  return p;
+}
+
+// Per-problem description of a batched (concatenated) site space: problem = segment.
 struct BatchSeg {
   const void* mat[3];   // D+ M5op^-1, M5op^-dag D+^dag, D+^dag in the accumulation type
   double l_alpha, l_beta, mf, db, dc;
   Coef5<double> k64;    // the same coefficients for the stage kernels (pre = 1)
   Coef5<float> k32;
+  Post5 post5;          // FP64 recurrence post (factor 1)
   int Vh;               // sites of one parity of this problem
   int first_tile;       // first 32-site tile of the problem in the concatenation
   int ntiles;

@@ -235,6 +235,15 @@ bool fifth_dim_matrices(int Ls, double M5, double mf, double b, double c,
                         std::vector<double>& dpm5i, std::vector<double>& m5idpt,
                         std::vector<double>& dpt, double* alpha, double* beta);
 
+// Multiprocessors of the current device (1 if the query fails).
+inline int sm_count() {
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0)
+    n = 1;
+  return n;
+}
+
 // Field sizes in bytes.
 inline size_t real_bytes(int prec) { return prec == P64 ? 8 : prec == P32 ? 4 : 2; }
 inline size_t field_bytes(const Geom& g, int prec) {

@@ -631,17 +631,18 @@ static dwf_status run_mspcg(dwf_ctx* h, Layout* lay, Layout* layL, int l, int in
   const Geom& g = layL->g;     // outer vectors
   const Geom& gb = lay->g;     // local solves
   const bool simd = use_simd_local(inner);
-  long max_ctas = std::max(g.Vp, gb.Vp) / 32;
+  // one partial per CTA: at the finest one site per CTA (FP64 stages)
+  long max_ctas = std::max(g.Vp, gb.Vp);
   if (exact && !simd) {
     // before the engines pack links: packing also gathers the halo copies
     DWF_TRY(ensure_halo(h, lay));
-    max_ctas = std::max(max_ctas, lay->halo->He_tot / 32);
+    max_ctas = std::max(max_ctas, lay->halo->He_tot);
   }
   OpEngine E64, Em, Ei;
   DWF_TRY(E64.init(h, layL, P64, false));
   DWF_TRY(Em.init(h, layL, middle, false));
   if (!simd) DWF_TRY(Ei.init(h, lay, inner, true));
-  DWF_TRY(ensure_reduction(h, max_ctas * 2 + 64, gb.nblocks + 64));
+  DWF_TRY(ensure_reduction(h, max_ctas + 64, gb.nblocks + 64));
   const size_t f64 = field_bytes(g, P64), fm = field_bytes(g, middle), fi = field_bytes(gb, inner);
   void *b64, *x64, *r64, *t1, *t2, *t3;
   DWF_TRY(h->ws->get("ms_b64", f64, &b64));
@@ -872,7 +873,7 @@ static dwf_status run_ms(dwf_ctx* h, Layout* lay, Layout* layL, int l, int inner
   const Geom& g = layL->g;
   OpEngine E64;
   DWF_TRY(E64.init(h, layL, P64, false));
-  DWF_TRY(ensure_reduction(h, g.Vp / 32 * 2 + 64, 64));
+  DWF_TRY(ensure_reduction(h, g.Vp + 64, 64));
   SimdLocal* S;
   DWF_TRY(ensure_simd(h, lay, exact, &S));
   const size_t f64 = field_bytes(g, P64);

@@ -61,6 +61,7 @@ struct StageArgs {
   float hs32;
   Coef5<double> k64;
   Coef5<float> k32;
+  Post5 post5;           // FP64 recurrence post, constants folded
   int epi;
   const double* alpha;   // EPI_CG_R: per-segment alpha
   int seg_cps;           // CTAs per scalar/reduction segment (Vp/32: one global segment)
@@ -83,9 +84,11 @@ template <typename A>
 __device__ __forceinline__ Coef5<A> coef5(const BatchSeg& S) {
   if constexpr (sizeof(A) == 8) return S.k64; else return S.k32;
 }
-inline void finish_stage_args(StageArgs& a, int Ls) {
+inline void finish_stage_args(StageArgs& a, int Ls, bool dag) {
   a.hs32 = (float)a.hop_scale;
   const double pre = a.post_pre != 0.0 ? a.post_pre : 1.0;
+  a.post5 = make_post5(a.l_alpha, a.l_beta, a.mf, a.dp_b, a.dp_c,
+                       a.hop_scale * (dag ? 1.0 : pre), Ls);
   a.k64 = make_coef5<double>(a.l_alpha, a.l_beta, a.mf, a.dp_b, a.dp_c, pre, Ls);
   a.k32 = make_coef5<float>(a.l_alpha, a.l_beta, a.mf, a.dp_b, a.dp_c, pre, Ls);
 }

@@ -28,7 +28,7 @@ static cudaError_t launch_stage_p(const StageArgs& a, int Ls, bool dag, bool blo
 cudaError_t launch_stage_prec(int prec, const StageArgs& args, int Ls, bool dag, bool blocked,
                               cudaStream_t st) {
   StageArgs a = args;
-  finish_stage_args(a, Ls);
+  finish_stage_args(a, Ls, dag);
   switch (prec) {
     case P64: return launch_stage_p<P64>(a, Ls, dag, blocked, st);
     case P32: return launch_stage_p<P32>(a, Ls, dag, blocked, st);

@@ -11,6 +11,7 @@
 #include <tuple>
 
 #include "dwf_internal.h"
+#include "stage64.cuh"
 
 namespace dwf {
 
@@ -68,7 +69,7 @@ struct StageTune {
 // L1-cached cp.async ring with a register budget for 2 or 3 CTAs per SM, with the tile's links
 // and streams prefetched into L2 or its links staged in shared memory by TMA, one CTA per tile
 // (persistent grids measured 10-35 % slower there; only the tensor-core post, whose set-up is
-// per CTA, has them).  FP32 and FP64 (ALU bound): one CTA per tile or a persistent grid.
+// per CTA, has them).  FP32: one CTA per tile or a persistent grid.
 template <int P, int LS, bool DAG, bool BLK, int POST, int MINB, int G, int SP = 1>
 static void stage_cand(StageCand* c, int& n, int per_sm) {
   c[n++] = {stage_launch_v<P, LS, DAG, BLK, POST, MINB, G, SP>,
@@ -94,7 +95,7 @@ static void stage_cands(StageCand* c, int& n) {
     stage_cand<P, LS, DAG, BLK, POST, 5 - MB, G_RING>(c, n, 0);
     stage_cand<P, LS, DAG, BLK, POST, MB, G_RING_BPF>(c, n, 0);
     stage_cand<P, LS, DAG, BLK, POST, MB, G_RING_TMA>(c, n, 0);
-  } else if constexpr (P == P32) {
+  } else {
     stage_cand<P, LS, DAG, BLK, POST, 2, G_BPF_L>(c, n, 0);
     stage_cand<P, LS, DAG, BLK, POST, 2, G_REG>(c, n, 0);
     stage_cand<P, LS, DAG, BLK, POST, 2, G_BPF_LS>(c, n, 0);
@@ -106,18 +107,7 @@ static void stage_cands(StageCand* c, int& n) {
     // the same with the pairs packed in float2 (f32x2 arithmetic)
     stage_cand<P, LS, DAG, BLK, POST, 2, G_TMA, SP_PAIR_F2>(c, n, 0);
     stage_cand<P, LS, DAG, BLK, POST, 2, G_TMA, SP_PAIR_F2>(c, n, 2);
-  } else {
-    stage_cand<P, LS, DAG, BLK, POST, 2, G_REG>(c, n, 0);
-    stage_cand<P, LS, DAG, BLK, POST, 2, G_REG>(c, n, 2);
   }
-}
-
-static int sm_count() {
-  int n = 0;
-  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, current_device()) !=
-          cudaSuccess || n <= 0)
-    n = 1;
-  return n;
 }
 
 template <int P, int LS, bool DAG, bool BLK>
@@ -226,10 +216,46 @@ static cudaError_t stage_launch_one(const StageArgs& a, cudaStream_t st) {
   return c[v].fn(b, c[v].smem, grid_of(c[v]), st);
 }
 
+// FP64 stages have one kernel, whose launch shape follows from the sizes (stage64.cuh).
+template <int LS, bool DAG, bool BLK, int POST, int DS>
+static cudaError_t stage64_launch(const StageArgs& a, int lst, cudaStream_t st) {
+  auto k = stage64_kernel<LS, DAG, BLK, POST, DS>;
+  const size_t sm = stage64_smem(LS, POST, 1 << lst, DS);
+  if (sm > 40 * 1024) {   // 48 KB without asking, static shared memory included
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+  }
+  k<<<dim3((unsigned)(a.ntiles * 32 >> lst)), dim3((unsigned)((LS << lst) * DS)), sm, st>>>(a, lst);
+  return cudaGetLastError();
+}
+template <int LS, bool DAG, bool BLK, int POST>
+static cudaError_t stage64_launch_ds(const StageArgs& a, cudaStream_t st) {
+  const Stage64Shape s = stage64_shape(a.ntiles * 32, LS, sm_count(), 8);
+  return s.ds == 8 ? stage64_launch<LS, DAG, BLK, POST, 8>(a, s.lst, st)
+                   : stage64_launch<LS, DAG, BLK, POST, 1>(a, s.lst, st);
+}
+template <int LS, bool DAG, bool BLK>
+static cudaError_t stage64_launch_post(const StageArgs& a, cudaStream_t st) {
+  if (a.wait_probe) return cudaErrorNotSupported;   // no TMA link staging
+  StageArgs b = a;
+  if (b.ntiles == 0) b.ntiles = b.Vp / 32;
+  if (!b.post) return stage64_launch_ds<LS, DAG, BLK, 0>(b, st);
+  if (b.post_sparse) {
+    if constexpr (DAG) return stage64_launch_ds<LS, DAG, BLK, 3>(b, st);
+    return cudaErrorInvalidValue;   // the sparse post is D+^dag, of adjoint stages only
+  }
+  return b.post_struct ? stage64_launch_ds<LS, DAG, BLK, 4>(b, st)
+                       : stage64_launch_ds<LS, DAG, BLK, 1>(b, st);
+}
+
 template <int P, int LS, bool DAG>
 cudaError_t stage_dispatch_ls(const StageArgs& a, bool blocked, cudaStream_t st) {
-  return blocked ? stage_launch_one<P, LS, DAG, true>(a, st)
-                 : stage_launch_one<P, LS, DAG, false>(a, st);
+  if constexpr (P == P64)
+    return blocked ? stage64_launch_post<LS, DAG, true>(a, st)
+                   : stage64_launch_post<LS, DAG, false>(a, st);
+  else
+    return blocked ? stage_launch_one<P, LS, DAG, true>(a, st)
+                   : stage_launch_one<P, LS, DAG, false>(a, st);
 }
 
 }  // namespace dwf

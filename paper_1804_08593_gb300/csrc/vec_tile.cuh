@@ -37,26 +37,31 @@ __device__ __forceinline__ void load_z_as(Spinor<typename Prec<P>::acc>& r, cons
   for (int k = 0; k < 12; k++) r.c[k] = {A((AW)v.c[k].x * fw), A((AW)v.c[k].y * fw)};
 }
 
-// The CG update of one 32-site tile (all Ls slices; thread (lane, s)); ntiles_all: the CTAs that
+// The CG update of one tile (all Ls slices; thread (lane, s)); ntiles_all: the CTAs that
 // count on the single-segment completion counter.  COH: inputs written earlier in the same
-// launch (persistent kernels) are read through L2.
+// launch (persistent kernels) are read through L2.  A tile is 32 sites; for FP64, where the
+// two FP64 lanes per clock and SM are what a small lattice waits for, it is blockDim.x sites
+// (a power of two up to 32), so that every SM gets some.
 template <int P, int LS, bool COH = false>
 __device__ __forceinline__ void vec_tile(const VecArgs& a, long tile, unsigned ntiles_all,
                                          unsigned char* smem_raw) {
   using A = typename Prec<P>::acc;
   const int lane = threadIdx.x, s = threadIdx.y;
-  const long site = tile * 32 + lane;
+  const int W = P == P64 ? (int)blockDim.x : 32;   // sites of a tile
+  const long site = tile * W + lane;
+  const long tile32 = P == P64 ? tile * W >> 5 : tile;
+  const int per = 32 / W;
   int seg;
   double dbv = a.db, dcv = a.dc, mfv = a.mf;
   if (a.tile_seg) {
-    seg = a.tile_seg[tile];
+    seg = a.tile_seg[tile32];
     if (a.stop && a.stop[seg]) return;
     dbv = a.segp[seg].db;
     dcv = a.segp[seg].dc;
     mfv = a.segp[seg].mf;
   } else {
     if (a.stop && *a.stop) return;
-    seg = (int)(tile / a.seg_cps);
+    seg = (int)(tile32 / a.seg_cps);
   }
 
   Spinor<A> p;
@@ -114,20 +119,20 @@ __device__ __forceinline__ void vec_tile(const VecArgs& a, long tile, unsigned n
     A* buf = reinterpret_cast<A*>(smem_raw);
 #pragma unroll
     for (int k = 0; k < 12; k++) {
-      buf[(s * 24 + 2 * k) * 32 + lane] = p.c[k].x;
-      buf[(s * 24 + 2 * k + 1) * 32 + lane] = p.c[k].y;
+      buf[(s * 24 + 2 * k) * W + lane] = p.c[k].x;
+      buf[(s * 24 + 2 * k + 1) * W + lane] = p.c[k].y;
     }
     __syncthreads();
     const int su = s + 1 < LS ? s + 1 : 0, sd = s > 0 ? s - 1 : LS - 1;
     const A fu = (s + 1 < LS) ? A(1) : A(-mfv), fd = (s > 0) ? A(1) : A(-mfv);
-    const A db = A(dbv), dc = A(dcv);
+    const A db = A(dbv), dc = A(dcv), cu = dc * fu, cd = dc * fd;
     Spinor<A> u;
 #pragma unroll
     for (int k = 0; k < 12; k++) {
       const int sn = k < 6 ? sd : su;
-      const A f = k < 6 ? fd : fu;
-      u.c[k].x = db * p.c[k].x + dc * f * buf[(sn * 24 + 2 * k) * 32 + lane];
-      u.c[k].y = db * p.c[k].y + dc * f * buf[(sn * 24 + 2 * k + 1) * 32 + lane];
+      const A f = k < 6 ? cd : cu;
+      u.c[k].x = db * p.c[k].x + f * buf[(sn * 24 + 2 * k) * W + lane];
+      u.c[k].y = db * p.c[k].y + f * buf[(sn * 24 + 2 * k + 1) * W + lane];
     }
     store_spinor<P>(a.u, a.Vp, site, s, u);
   }
@@ -136,7 +141,7 @@ __device__ __forceinline__ void vec_tile(const VecArgs& a, long tile, unsigned n
     if (a.tile_seg) {
       // per problem: the last tile of the problem copies its convergence flag to its stop
       // flag and counts the iteration
-      if (last_cta(a.red.counter + seg, a.segp[seg].ntiles) && tid == 0) {
+      if (last_cta(a.red.counter + seg, a.segp[seg].ntiles * per) && tid == 0) {
         if (a.stop_out && a.conv_in && a.conv_in[seg]) a.stop_out[seg] = 1;
         if (a.iter) a.iter[seg] += 1;
         a.red.counter[seg] = 0u;

@@ -180,3 +180,38 @@ def test_every_launch_variant_matches_oracle(variant, prec, monkeypatch):
         out = cuda(np.zeros_like(x))
         dwf.dwf_apply(h, op, cuda(x), out, prec)
         assert rel(host(out), ref) <= TOL[prec], (variant, op, rel(host(out), ref))
+
+
+@pytest.mark.parametrize("dims,Ls", [((2, 2, 2, 2), 4), ((2, 2, 2, 2), 16), ((6, 6, 6, 10), 10),
+                                     ((6, 6, 6, 10), 6), ((8, 8, 8, 8), 12), ((8, 8, 8, 8), 4),
+                                     ((10, 8, 6, 10), 16)])
+def test_fp64_stage_shapes(dims, Ls):
+    """FP64 stages choose sites per CTA and whole hops or direction groups by size: the
+    smallest lattices of each, ragged ones, and sizes on both sides of the choice."""
+    dwf = lib()
+    rng, U, p = _setup((dims, Ls, 1.8, 0.07, 1.5, 0.5, 0.3), 17)
+    h = dwf.dwf_create(p.dims, p.Ls, p.M5, p.mf, p.b, p.c, cuda(U))
+    x = rand_even(rng, p.dims, p.Ls)
+    out = cuda(np.zeros_like(x))
+    for op, ref in (("Mpc", o.mpc(U, x, p)), ("MdagM", o.mdagm(U, x, p))):
+        dwf.dwf_apply(h, op, cuda(x), out, "f64")
+        assert rel(host(out), ref) <= TOL["f64"], (op, rel(host(out), ref))
+
+
+@pytest.mark.parametrize("local_op", [0, 1])
+def test_fp64_blocked_stages_match_the_persistent_local_solver(local_op, monkeypatch):
+    """Blocked FP64 stages with whole hops (4096 even sites): three outer steps of MSPCG agree
+    with the persistent local solver's.  Both are FP64 throughout; 1e-10 leaves the rounding
+    differences of 3 x 2 CG steps a factor of 1e5."""
+    dwf = lib()
+    rng, U, p = _setup(((8, 8, 8, 16), 8, 1.8, 0.1, 1.5, 0.5, 0.3), 19)
+    phi = cuda(rand_even(rng, p.dims, p.Ls))
+    x = {}
+    for solver in ("stages", "persistent"):
+        monkeypatch.setenv("DWF_LOCAL_SOLVER", solver)
+        h = dwf.dwf_create(p.dims, p.Ls, p.M5, p.mf, p.b, p.c, cuda(U))
+        out = cuda(np.zeros(phi.shape, complex))
+        dwf.dwf_mspcg(h, (4, 4, 4, 4), 2, "f64", "f64", phi, out, 1e-10, 3, local_op=local_op,
+                      raise_on_fail=False)
+        x[solver] = host(out)
+    assert rel(x["stages"], x["persistent"]) <= 1e-10
