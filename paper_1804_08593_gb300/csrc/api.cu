@@ -232,20 +232,20 @@ dwf_status dwf_apply(dwf_t h, dwf_op op, const void* in, void* out, dwf_prec pre
       DWF_TRY(unpack_full(h, lay, e, f, prec, dout));
       break;
     case DWF_OP_MPC:
-      DWF_TRY(pack_even(h, lay, din, a, prec, 1.0));
+      DWF_TRY(pack_even(h, lay, din, a, prec));
       DWF_TRY(E.mpc(a, b, c, d, EPI_STORE, none, nullptr));
-      DWF_TRY(unpack_even(h, lay, d, prec, dout, 1.0));
+      DWF_TRY(unpack_even(h, lay, d, prec, dout));
       break;
     case DWF_OP_MPC_DAG:
-      DWF_TRY(pack_even(h, lay, din, a, prec, 1.0));
+      DWF_TRY(pack_even(h, lay, din, a, prec));
       DWF_TRY(E.mpcdag(a, c, d, EPI_STORE, nullptr, nullptr, none, nullptr));
-      DWF_TRY(unpack_even(h, lay, d, prec, dout, 1.0));
+      DWF_TRY(unpack_even(h, lay, d, prec, dout));
       break;
     case DWF_OP_MDAGM:
-      DWF_TRY(pack_even(h, lay, din, a, prec, 1.0));
+      DWF_TRY(pack_even(h, lay, din, a, prec));
       DWF_TRY(E.mpc(a, b, c, d, EPI_STORE, none, nullptr));
       DWF_TRY(E.mpcdag(d, c, e, EPI_STORE, nullptr, nullptr, none, nullptr));
-      DWF_TRY(unpack_even(h, lay, e, prec, dout, 1.0));
+      DWF_TRY(unpack_even(h, lay, e, prec, dout));
       break;
     default:
       return set_error(DWF_ERR_ARG, "unknown operator");

@@ -251,11 +251,8 @@ inline size_t field_bytes(const Geom& g, int prec) {
 }
 
 // Caller even-half c128 (device) <-> internal even field of precision prec.
-// scale: multiplies on pack, divides on unpack (FP16/BF16 range control).
-dwf_status pack_even(dwf_ctx* h, Layout* lay, const void* src_c128, void* dst, int prec,
-                     double scale);
-dwf_status unpack_even(dwf_ctx* h, Layout* lay, const void* src, int prec, void* dst_c128,
-                       double scale);
+dwf_status pack_even(dwf_ctx* h, Layout* lay, const void* src_c128, void* dst, int prec);
+dwf_status unpack_even(dwf_ctx* h, Layout* lay, const void* src, int prec, void* dst_c128);
 // Caller full c128 <-> internal (even, odd) fields.
 dwf_status pack_full(dwf_ctx* h, Layout* lay, const void* src_c128, void* dst_even,
                      void* dst_odd, int prec);

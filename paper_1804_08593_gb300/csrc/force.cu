@@ -163,7 +163,7 @@ extern "C" dwf_status dwf_force(dwf_t h, const void* phi, const void* X, void* d
   DWF_TRY(h->ws->get("force_w", fb, &w));
   DWF_TRY(h->ws->get("force_y", fb, &y));
   DWF_TRY(h->ws->get("force_z", fb, &z));
-  DWF_TRY(pack_even(h, lay, dX, x, P64, 1.0));
+  DWF_TRY(pack_even(h, lay, dX, x, P64));
   // Y = Mpc X; the first stage leaves W = D+ M5op^-1 Dh_oe D+ X in w and D+ X in u
   DWF_TRY(E.mpc(x, u, w, y, EPI_STORE, RedArgs{}, nullptr));
   const void* V = x;
@@ -235,8 +235,8 @@ extern "C" dwf_status dwf_action(dwf_t h, const void* phi, const void* X, double
   DWF_TRY(h->ws->get("force_w", fb, &t));
   DWF_TRY(h->ws->get("force_y", fb, &y));
   DWF_TRY(h->ws->get("force_d", 4 * sizeof(double), (void**)&d));
-  DWF_TRY(pack_even(h, lay, dX, x, P64, 1.0));
-  DWF_TRY(pack_even(h, lay, dphi, f, P64, 1.0));
+  DWF_TRY(pack_even(h, lay, dX, x, P64));
+  DWF_TRY(pack_even(h, lay, dphi, f, P64));
   // S = Re(2 <phi, X> - ||Mpc X||^2): equals phi^dag A^-1 phi at the exact solution, with an
   // error quadratic in the solve residual.
   DWF_TRY(E.mpc(x, u, t, y, EPI_NORM, E.red(FIN_STORE, d), nullptr));

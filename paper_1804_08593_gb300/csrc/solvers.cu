@@ -248,8 +248,8 @@ static dwf_status run_cg(dwf_ctx* h, Layout* lay, const void* b_c128, void* x_c1
   if (hcap && stats->curvature_history)
     DWF_TRY(h->ws->get("cg_curv", (size_t)hcap * sizeof(double), (void**)&dcurv));
 
-  DWF_TRY(pack_even(h, lay, b_c128, b64, P64, 1.0));
-  if (x0) DWF_TRY(pack_even(h, lay, x_c128, x64, P64, 1.0));
+  DWF_TRY(pack_even(h, lay, b_c128, b64, P64));
+  if (x0) DWF_TRY(pack_even(h, lay, x_c128, x64, P64));
   else DWF_TRY(vop(E64, VOP_ZERO, nullptr, x64));
 
   double bb, rr;
@@ -258,7 +258,7 @@ static dwf_status run_cg(dwf_ctx* h, Layout* lay, const void* b_c128, void* x_c1
   if (!(bb > 0.0) || !std::isfinite(bb)) {
     if (bb == 0.0) {  // zero source: zero solution
       DWF_TRY(vop(E64, VOP_ZERO, nullptr, x64));
-      DWF_TRY(unpack_even(h, lay, x64, P64, x_c128, 1.0));
+      DWF_TRY(unpack_even(h, lay, x64, P64, x_c128));
       DWF_CUDA(cudaStreamSynchronize(h->stream));
       if (stats) stats->seconds = timer.seconds();
       return DWF_OK;
@@ -351,7 +351,7 @@ static dwf_status run_cg(dwf_ctx* h, Layout* lay, const void* b_c128, void* x_c1
       stats->operator_applications++;
     }
   }
-  DWF_TRY(unpack_even(h, lay, x64, P64, x_c128, 1.0));
+  DWF_TRY(unpack_even(h, lay, x64, P64, x_c128));
   DWF_CUDA(cudaStreamSynchronize(h->stream));
   if (stats) {
     stats->iterations = iters;
@@ -698,13 +698,13 @@ static dwf_status run_mspcg(dwf_ctx* h, Layout* lay, Layout* layL, int l, int in
   DWF_TRY(h->ws->get("ms_blk", 5 * (size_t)gb.nblocks * sizeof(double), (void**)&blk));
   DWF_CUDA(cudaMemsetAsync(dsc, 0, S_NSLOT * sizeof(double), h->stream));
 
-  DWF_TRY(pack_even(h, layL, b_c128, b64, P64, 1.0));
+  DWF_TRY(pack_even(h, layL, b_c128, b64, P64));
   DWF_TRY(vop(E64, VOP_ZERO, nullptr, x64));
   double bb, rr64, rrm;
   DWF_TRY(true_residual(E64, b64, nullptr, r64, t1, t2, t3, dsc, &bb));
   if (!(bb > 0.0) || !std::isfinite(bb)) {
     if (bb == 0.0) {
-      DWF_TRY(unpack_even(h, layL, x64, P64, x_c128, 1.0));
+      DWF_TRY(unpack_even(h, layL, x64, P64, x_c128));
       DWF_CUDA(cudaStreamSynchronize(h->stream));
       return DWF_OK;
     }
@@ -813,7 +813,7 @@ static dwf_status run_mspcg(dwf_ctx* h, Layout* lay, Layout* layL, int l, int in
     DWF_TRY(vop(E64, VOP_ADD_CAST, xm, x64, RedArgs{}, 1.0, nullptr, middle));
     DWF_TRY(true_residual(E64, b64, x64, r64, t1, t2, t3, dsc, &rr64));
   }
-  DWF_TRY(unpack_even(h, layL, x64, P64, x_c128, 1.0));
+  DWF_TRY(unpack_even(h, layL, x64, P64, x_c128));
   DWF_CUDA(cudaStreamSynchronize(h->stream));
   if (stats) {
     stats->iterations = k;
@@ -895,13 +895,13 @@ static dwf_status run_ms(dwf_ctx* h, Layout* lay, Layout* layL, int l, int inner
   DWF_TRY(h->ws->get("ms_yi", per * S->sE, &F.y));
   double* dsc;
   DWF_TRY(h->ws->get("ms_scal", S_NSLOT * sizeof(double), (void**)&dsc));
-  DWF_TRY(pack_even(h, layL, b_c128, b64, P64, 1.0));
+  DWF_TRY(pack_even(h, layL, b_c128, b64, P64));
   DWF_TRY(vop(E64, VOP_ZERO, nullptr, x64));
   double bb, rr;
   DWF_TRY(true_residual(E64, b64, nullptr, r64, t1, t2, t3, dsc, &bb));
   if (!(bb > 0.0) || !std::isfinite(bb)) {
     if (bb == 0.0) {
-      DWF_TRY(unpack_even(h, layL, x64, P64, x_c128, 1.0));
+      DWF_TRY(unpack_even(h, layL, x64, P64, x_c128));
       DWF_CUDA(cudaStreamSynchronize(h->stream));
       return DWF_OK;
     }
@@ -934,7 +934,7 @@ static dwf_status run_ms(dwf_ctx* h, Layout* lay, Layout* layL, int l, int inner
   }
   if (rr <= tol * tol * bb) status = DWF_OK;
   DWF_TRY(check_device_error(h));
-  DWF_TRY(unpack_even(h, layL, x64, P64, x_c128, 1.0));
+  DWF_TRY(unpack_even(h, layL, x64, P64, x_c128));
   DWF_CUDA(cudaStreamSynchronize(h->stream));
   if (stats) {
     stats->iterations = k;

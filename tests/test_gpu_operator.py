@@ -215,3 +215,30 @@ def test_fp64_blocked_stages_match_the_persistent_local_solver(local_op, monkeyp
                       raise_on_fail=False)
         x[solver] = host(out)
     assert rel(x["stages"], x["persistent"]) <= 1e-10
+
+
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (4, 6, 2, 6)])
+def test_single_precision_rounding_of_caller_fields(dims):
+    """With zero links and M5 = 4 the operator leaves slice 0 of a source on slice 0 as it is, so
+    an FP32 application returns the source rounded to FP32: compared bit for bit with numpy's
+    conversion at ties, over the FP32 range and in its subnormals.  (Up to 2^125: the hop adds two
+    components, and an overflow there times a zero link is a NaN.)"""
+    dwf = lib()
+    Ls, n = 4, dims[0] * dims[1] * dims[2] * dims[3] // 2 * 24
+    U = np.zeros((dims[3], dims[2], dims[1], dims[0], 4, 3, 3), complex)
+    rng = np.random.default_rng(23)
+    f = np.ldexp(rng.uniform(1.0, 2.0, n), rng.integers(-152, 125, n)) * rng.choice([-1.0, 1.0], n)
+    tie = np.float32(f).astype(np.float64)
+    ulp = np.spacing(np.abs(np.float32(f))).astype(np.float64)
+    f[0::4] = tie[0::4] + 0.5 * ulp[0::4]          # exact ties
+    f[1::4] = np.nextafter(tie[1::4] + 0.5 * ulp[1::4], 0.0)
+    f[2::8] = tie[2::8]
+    f[:8] = [0.0, -0.0, 2.0 ** -126, 2.0 ** -149, 2.0 ** -150, 2.0 ** -126 * (1 - 2.0 ** -30),
+             2.0 ** 125 * (1 + 2.0 ** -24), -2.0 ** 125 * (1 + 3 * 2.0 ** -24)]
+    x = np.zeros((Ls, n // 24, 4, 3), complex)
+    x[0] = f.reshape(-1, 2).view(complex).reshape(n // 24, 4, 3)
+    h = dwf.dwf_create(dims, Ls, 4.0, 0.1, 1.0, 0.0, cuda(U))
+    out = cuda(np.zeros_like(x))
+    dwf.dwf_apply(h, "Mpc", cuda(x), out, "f32")
+    got = np.ascontiguousarray(host(out)[0]).reshape(-1).view(float)
+    assert np.array_equal(got, np.float32(f).astype(np.float64))
