@@ -225,14 +225,98 @@ __device__ __forceinline__ void hop_acc_out(const HopAcc<P>& h,
   }
 }
 
+// One hop term for a pair of slices, component k of both in one float2 (f32x2 arithmetic, each
+// link element broadcast to both halves).  The sign of gamma is a runtime value, +-1 multiplied
+// inside the FMAs that add (the same roundings), so that Dh and Dh^dag share one copy of the
+// code: with four unrolled copies (one per hop phase, 150 KB) the kernel waited for
+// instructions (12^3x24, 32 blocks of 6^4, Ls = 12, l = 6: 1.63 ms a launch, now 1.40; 24^4,
+// 256 blocks: 7.21, now 7.19, where three CTAs per SM hide the rest).
+template <int MU>
+__device__ __forceinline__ void hop_term_f2s(cx2 (&acc)[12], const Spinor<float>& psi0,
+                                             const Spinor<float>& psi1, const cx<float> (&u)[9],
+                                             float sgn) {
+  const float2 m1 = bcast2(-1.f), sp = bcast2(sgn), sm = bcast2(-sgn);
+  // h = psi_up + sgn B psi_dn on the pairs
+  auto pair = [&](int k) -> cx2 {
+    return {make_float2(psi0.c[k].x, psi1.c[k].x), make_float2(psi0.c[k].y, psi1.c[k].y)};
+  };
+  cx2 h[2][3];
+#pragma unroll
+  for (int c = 0; c < 3; c++) {
+    const cx2 p0 = pair(c), p1 = pair(3 + c), p2 = pair(6 + c), p3 = pair(9 + c);
+    if constexpr (MU == 0) {          // -i p3, -i p2
+      h[0][c] = {__ffma2_rn(p3.y, sp, p0.x), __ffma2_rn(p3.x, sm, p0.y)};
+      h[1][c] = {__ffma2_rn(p2.y, sp, p1.x), __ffma2_rn(p2.x, sm, p1.y)};
+    } else if constexpr (MU == 1) {   // -p3, p2
+      h[0][c] = {__ffma2_rn(p3.x, sm, p0.x), __ffma2_rn(p3.y, sm, p0.y)};
+      h[1][c] = {__ffma2_rn(p2.x, sp, p1.x), __ffma2_rn(p2.y, sp, p1.y)};
+    } else if constexpr (MU == 2) {   // -i p2, i p3
+      h[0][c] = {__ffma2_rn(p2.y, sp, p0.x), __ffma2_rn(p2.x, sm, p0.y)};
+      h[1][c] = {__ffma2_rn(p3.y, sm, p1.x), __ffma2_rn(p3.x, sp, p1.y)};
+    } else {                          // p2, p3
+      h[0][c] = {__ffma2_rn(p2.x, sp, p0.x), __ffma2_rn(p2.y, sp, p0.y)};
+      h[1][c] = {__ffma2_rn(p3.x, sp, p1.x), __ffma2_rn(p3.y, sp, p1.y)};
+    }
+  }
+#pragma unroll
+  for (int a = 0; a < 3; a++) {
+    const float2 ux0 = bcast2(u[3 * a].x), uy0 = bcast2(u[3 * a].y);
+    const float2 ux1 = bcast2(u[3 * a + 1].x), uy1 = bcast2(u[3 * a + 1].y);
+    const float2 ux2 = bcast2(u[3 * a + 2].x), uy2 = bcast2(u[3 * a + 2].y);
+    cx2 g[2];
+#pragma unroll
+    for (int i = 0; i < 2; i++) {
+      float2 re = __fmul2_rn(ux0, h[i][0].x);
+      re = __ffma2_rn(ux1, h[i][1].x, re);
+      re = __ffma2_rn(ux2, h[i][2].x, re);
+      float2 q = __fmul2_rn(uy0, h[i][0].y);
+      q = __ffma2_rn(uy1, h[i][1].y, q);
+      q = __ffma2_rn(uy2, h[i][2].y, q);
+      float2 im = __fmul2_rn(ux0, h[i][0].y);
+      im = __ffma2_rn(ux1, h[i][1].y, im);
+      im = __ffma2_rn(ux2, h[i][2].y, im);
+      im = __ffma2_rn(uy0, h[i][0].x, im);
+      im = __ffma2_rn(uy1, h[i][1].x, im);
+      im = __ffma2_rn(uy2, h[i][2].x, im);
+      g[i] = {__ffma2_rn(q, m1, re), im};
+    }
+    auto add = [&](float2& c, float2 v, float2 f) { c = __ffma2_rn(v, f, c); };
+    acc[a] = {__fadd2_rn(acc[a].x, g[0].x), __fadd2_rn(acc[a].y, g[0].y)};
+    acc[3 + a] = {__fadd2_rn(acc[3 + a].x, g[1].x), __fadd2_rn(acc[3 + a].y, g[1].y)};
+    // lower spins: sgn * B^dag g (i z = (-z.y, z.x))
+    if constexpr (MU == 0) {          // i g1, i g0
+      add(acc[6 + a].x, g[1].y, sm);
+      add(acc[6 + a].y, g[1].x, sp);
+      add(acc[9 + a].x, g[0].y, sm);
+      add(acc[9 + a].y, g[0].x, sp);
+    } else if constexpr (MU == 1) {   // g1, -g0
+      add(acc[6 + a].x, g[1].x, sp);
+      add(acc[6 + a].y, g[1].y, sp);
+      add(acc[9 + a].x, g[0].x, sm);
+      add(acc[9 + a].y, g[0].y, sm);
+    } else if constexpr (MU == 2) {   // i g0, -i g1
+      add(acc[6 + a].x, g[0].y, sm);
+      add(acc[6 + a].y, g[0].x, sp);
+      add(acc[9 + a].x, g[1].y, sp);
+      add(acc[9 + a].y, g[1].x, sm);
+    } else {                          // g0, g1
+      add(acc[6 + a].x, g[0].x, sp);
+      add(acc[6 + a].y, g[0].y, sp);
+      add(acc[9 + a].x, g[1].x, sp);
+      add(acc[9 + a].y, g[1].y, sp);
+    }
+  }
+}
+
 // One hop direction D for the thread's slices: spinors from the chunks at q (slice j at
-// q + j * jstride, chunk k at + k * qs), the link from the tile's raw copy.
-template <int P, bool DAG, int D>
+// q + j * jstride, chunk k at + k * qs), the link from the tile's raw copy; fs: the sign of
+// gamma in forward hops, -1 (Dh) or +1 (Dh^dag), opposite in backward hops.
+template <int P, int D>
 __device__ __forceinline__ void simd_term(HopAcc<P>& acc, const uint4* q, int qs, int jstride,
-                                          const uint4* lraw, int lane) {
+                                          const uint4* lraw, int lane,
+                                          typename Prec<P>::acc fs) {
   using A = typename Prec<P>::acc;
-  constexpr bool back = (D & 1) != 0;
-  const A sgn = (back != DAG) ? A(1) : A(-1);
+  const A sgn = (D & 1) != 0 ? -fs : fs;
   cx<A> u[9];
   load_link9<P, true>(u, lraw, 32, lane, D);
   if constexpr (P == P64) {
@@ -243,22 +327,23 @@ __device__ __forceinline__ void simd_term(HopAcc<P>& acc, const uint4* q, int qs
     Spinor<float> psi0, psi1;
     unpack_chunks<P>(psi0, q, qs);
     unpack_chunks<P>(psi1, q + jstride, qs);
-    hop_term_f2<D / 2>(acc.c, psi0, psi1, u, sgn);
+    hop_term_f2s<D / 2>(acc.c, psi0, psi1, u, sgn);
   }
 }
 
-template <int P, bool DAG>
+template <int P>
 __device__ __forceinline__ void simd_term_d(int d, HopAcc<P>& acc, const uint4* q, int qs,
-                                            int jstride, const uint4* lraw, int lane) {
+                                            int jstride, const uint4* lraw, int lane,
+                                            typename Prec<P>::acc fs) {
   switch (d) {
-    case 0: simd_term<P, DAG, 0>(acc, q, qs, jstride, lraw, lane); break;
-    case 1: simd_term<P, DAG, 1>(acc, q, qs, jstride, lraw, lane); break;
-    case 2: simd_term<P, DAG, 2>(acc, q, qs, jstride, lraw, lane); break;
-    case 3: simd_term<P, DAG, 3>(acc, q, qs, jstride, lraw, lane); break;
-    case 4: simd_term<P, DAG, 4>(acc, q, qs, jstride, lraw, lane); break;
-    case 5: simd_term<P, DAG, 5>(acc, q, qs, jstride, lraw, lane); break;
-    case 6: simd_term<P, DAG, 6>(acc, q, qs, jstride, lraw, lane); break;
-    default: simd_term<P, DAG, 7>(acc, q, qs, jstride, lraw, lane); break;
+    case 0: simd_term<P, 0>(acc, q, qs, jstride, lraw, lane, fs); break;
+    case 1: simd_term<P, 1>(acc, q, qs, jstride, lraw, lane, fs); break;
+    case 2: simd_term<P, 2>(acc, q, qs, jstride, lraw, lane, fs); break;
+    case 3: simd_term<P, 3>(acc, q, qs, jstride, lraw, lane, fs); break;
+    case 4: simd_term<P, 4>(acc, q, qs, jstride, lraw, lane, fs); break;
+    case 5: simd_term<P, 5>(acc, q, qs, jstride, lraw, lane, fs); break;
+    case 6: simd_term<P, 6>(acc, q, qs, jstride, lraw, lane, fs); break;
+    default: simd_term<P, 7>(acc, q, qs, jstride, lraw, lane, fs); break;
   }
 }
 
@@ -267,10 +352,11 @@ __device__ __forceinline__ void simd_term_d(int d, HopAcc<P>& acc, const uint4* 
 // spinors go through a two-slot cp.async ring in shared memory, so the copy of the next live
 // direction is in flight while the current one is computed (each thread reads back only its
 // own copies: no block barrier).
-template <int P, int LS, bool DAG, int RS>
+template <int P, int LS, int RS>
 __device__ __forceinline__ void simd_hop(HopAcc<P>& acc, const uint32_t* row, uint32_t live,
                                          const void* in, long stride, int NB, long eg, int w,
-                                         const uint4* lraw, uint4* ring, int lane, int tid) {
+                                         const uint4* lraw, uint4* ring, int lane, int tid,
+                                         typename Prec<P>::acc fs) {
   constexpr int NCH = Prec<P>::NCH;
   constexpr int NSL = simd_nsl<P>();
   constexpr int LSP = LS / NSL;
@@ -284,7 +370,7 @@ __device__ __forceinline__ void simd_hop(HopAcc<P>& acc, const uint32_t* row, ui
       uint4 v[NCH];
 #pragma unroll
       for (int k = 0; k < NCH; k++) v[k] = __ldcg(q + k * stride);
-      simd_term_d<P, DAG>(d, acc, v, 1, 0, lraw, lane);
+      simd_term_d<P>(d, acc, v, 1, 0, lraw, lane, fs);
     }
   } else {
     // ring slot layout: [slot][slice j][chunk k][thread]; RS slots keep RS - 1 directions in
@@ -317,20 +403,21 @@ __device__ __forceinline__ void simd_hop(HopAcc<P>& acc, const uint32_t* row, ui
       else if (newer == 1) cp_async_wait<1>();
       else cp_async_wait<0>();
       const uint4* q = ring + ((i % RS) * NSL * NCH) * NT + tid;
-      simd_term_d<P, DAG>(nth(i), acc, q, NT, NCH * NT, lraw, lane);
+      simd_term_d<P>(nth(i), acc, q, NT, NCH * NT, lraw, lane, fs);
     }
   }
 }
 
 // The hop of the tile, unpacked into one spinor per slice of the thread.
-template <int P, int LS, bool DAG, int RS>
+template <int P, int LS, int RS>
 __device__ __forceinline__ void simd_hop_out(Spinor<typename Prec<P>::acc> (&out)[simd_nsl<P>()],
                                              const uint32_t* row, uint32_t live, const void* in,
                                              long stride, int NB, long eg, int w,
-                                             const uint4* lraw, uint4* ring, int lane, int tid) {
+                                             const uint4* lraw, uint4* ring, int lane, int tid,
+                                             typename Prec<P>::acc fs) {
   HopAcc<P> h;
   hop_acc_zero<P>(h);
-  simd_hop<P, LS, DAG, RS>(h, row, live, in, stride, NB, eg, w, lraw, ring, lane, tid);
+  simd_hop<P, LS, RS>(h, row, live, in, stride, NB, eg, w, lraw, ring, lane, tid, fs);
   hop_acc_out<P, simd_nsl<P>()>(h, out);
 }
 
@@ -627,6 +714,9 @@ simd_local_kernel(const SimdArgs a) {
   A* buf = reinterpret_cast<A*>(region);            // afterwards
   __shared__ A red[LSP][32];
   __shared__ double sc[32];
+  // the CG scalars of the lanes' blocks, kept out of the registers that the hop needs
+  __shared__ double rho_s[32];
+  __shared__ A alpha_s[32], beta_s[32];
   const int lane = threadIdx.x, w = threadIdx.y, tid = lane + 32 * w;
   const int C = a.C, slot = blockIdx.x % a.nslots, ci = blockIdx.x / a.nslots;
   if (slot >= a.nslots) return;
@@ -676,7 +766,6 @@ simd_local_kernel(const SimdArgs a) {
   for (int g = slot; g < a.ngroups; g += a.nslots) {
     const long eg0 = (long)g * 32;
     const long eg = eg0 + lane;   // this lane's block, as an element offset
-    double rho, alpha = 0.0, beta = 0.0;
     // this lane's block takes part in this call (Schwarz colour)
     bool active = true;
     if (a.ncol > 1) {
@@ -733,133 +822,122 @@ simd_local_kernel(const SimdArgs a) {
       }
       write_partial<A, LSP>(nrm, red, part + ci * 32, w, lane);
       if (!barrier()) return;
-      rho = slot_total(part, C, sc, w, lane);
+      const double tot = slot_total(part, C, sc, w, lane);
+      if (w == 0) rho_s[lane] = tot;
     }
     for (int k = 0; k < a.l; k++) {
       const bool last = (k + 1 == a.l);
-      // ---- P1: t = [D+ M5op^-1] Dh_oe (D+ p) on O
-      phase(a.sch[0], a.nsch[0], a.nbrO, a.linksO, sO, eg0,
-            [&](int pos, const uint32_t* row, uint32_t live, const uint4* lraw) {
-              Spinor<A> acc[NSL];
-              simd_hop_out<P, LS, false, RS>(acc, row, live, pin1, sB, NB, eg, w, lraw, ring, lane, tid);
-              __syncthreads();   // the ring becomes the post buffer
+      // ---- P1-P4 in one loop: the four hop phases run the same copy of the hop code (four
+      // copies did not fit the instruction caches)
+      bool done = false;
+#pragma unroll 1
+      for (int ph = 0; ph < 4; ph++) {
+        if (ph == 2 && last) {
+          // x += alpha p (the last iteration needs no new residual or direction)
+          const A al = alpha_s[lane];
+          for (int pos = ci; pos < a.nBE; pos += C) {
+            const long e = (long)pos * NB + eg;
 #pragma unroll
-              for (int j = 0; j < NSL; j++) to_buf(buf, acc[j], w + j * LSP, lane);
-              __syncthreads();
-              post_recurrence<A, LS, false>(buf, K, tid, NT);
-              __syncthreads();
+            for (int j = 0; j < NSL; j++) {
+              const int s = w + j * LSP;
+              Spinor<A> xv, pv;
+              ld_spinor<P>(xv, a.x, sB, e, s);
+              ld_spinor<P>(pv, a.p, sB, e, s);
 #pragma unroll
-              for (int j = 0; j < NSL; j++) {
-                from_buf(acc[j], buf, w + j * LSP, lane);
-                store_spinor<P>(a.t, sO, (long)pos * NB + eg, w + j * LSP, acc[j]);
+              for (int q = 0; q < 12; q++) {
+                xv.c[q].x += al * pv.c[q].x;
+                xv.c[q].y += al * pv.c[q].y;
               }
-            });
-      if (!barrier()) return;
-      // ---- P2: y = M5op p - 1/4 Dh_eo t on E; <p, A_s p> = ||y||^2 over the block
-      {
-        A nrm = A(0);
-        const A hs = A(-0.25);
-        phase(a.sch[1], a.nsch[1], a.nbrE, a.linksE, sE, eg0,
-              [&](int pos, const uint32_t* row, uint32_t live, const uint4* lraw) {
-                Spinor<A> acc[NSL];
-                simd_hop_out<P, LS, false, RS>(acc, row, live, a.t, sO, NB, eg, w, lraw, ring, lane,
-                                           tid);
-                const long e = (long)pos * NB + eg;
-#pragma unroll
-                for (int j = 0; j < NSL; j++) {
-                  const int s = w + j * LSP;
-#pragma unroll
-                  for (int q = 0; q < 12; q++) acc[j].c[q] = cscale(hs, acc[j].c[q]);
-                  if (pos < a.nBE) add_m5<P, false>(acc[j], a.p, sB, e, s, LS, K);
-                  nrm += norm2(acc[j]);
-                  if (!last) store_spinor<P>(a.y, sE, e, s, acc[j]);
-                }
-              });
-        write_partial<A, LSP>(nrm, red, part + ci * 32, w, lane);
-        if (!barrier()) return;
-        const double pap = slot_total(part, C, sc, w, lane);
-        alpha = (pap > 0.0 && isfinite(pap)) ? rho / pap : 0.0;
-      }
-      if (last) {
-        // ---- x += alpha p (the last iteration needs no new residual or direction)
-        const A al = A(alpha);
-        for (int pos = ci; pos < a.nBE; pos += C) {
-          const long e = (long)pos * NB + eg;
-#pragma unroll
-          for (int j = 0; j < NSL; j++) {
-            const int s = w + j * LSP;
-            Spinor<A> xv, pv;
-            ld_spinor<P>(xv, a.x, sB, e, s);
-            ld_spinor<P>(pv, a.p, sB, e, s);
-#pragma unroll
-            for (int q = 0; q < 12; q++) {
-              xv.c[q].x += al * pv.c[q].x;
-              xv.c[q].y += al * pv.c[q].y;
+              store_spinor<P>(a.x, sB, e, s, xv);
             }
-            store_spinor<P>(a.x, sB, e, s, xv);
           }
+          done = true;
+          break;
         }
-        break;
-      }
-      // ---- P3: s = [M5op^-dag D+^dag] Dh_oe^dag y on O
-      phase(a.sch[2], a.nsch[2], a.nbrO, a.linksO, sO, eg0,
-            [&](int pos, const uint32_t* row, uint32_t live, const uint4* lraw) {
-              Spinor<A> acc[NSL];
-              simd_hop_out<P, LS, true, RS>(acc, row, live, a.y, sE, NB, eg, w, lraw, ring, lane, tid);
-              __syncthreads();
-#pragma unroll
-              for (int j = 0; j < NSL; j++) to_buf(buf, acc[j], w + j * LSP, lane);
-              __syncthreads();
-              post_recurrence<A, LS, true>(buf, K, tid, NT);
-              __syncthreads();
-#pragma unroll
-              for (int j = 0; j < NSL; j++) {
-                from_buf(acc[j], buf, w + j * LSP, lane);
-                store_spinor<P>(a.t, sO, (long)pos * NB + eg, w + j * LSP, acc[j]);
-              }
-            });
-      if (!barrier()) return;
-      // ---- P4: r -= alpha (M5op^dag y - 1/4 D+^dag Dh_eo^dag s) on BE; ||r||^2 -> beta
-      {
+        const bool dag = ph >= 2, on_o = (ph & 1) == 0;
+        const void* in = ph == 0 ? pin1 : ph == 2 ? a.y : a.t;
+        const long in_s = ph == 0 ? sB : ph == 2 ? sE : sO;
+        const A fs = dag ? A(1) : A(-1);
         A nrm = A(0);
-        const A al = A(alpha), hs = A(a.hs_b);
-        phase(a.sch[3], a.nsch[3], a.nbrE, a.linksE, sE, eg0,
+        phase(a.sch[ph], a.nsch[ph], on_o ? a.nbrO : a.nbrE, on_o ? a.linksO : a.linksE,
+              on_o ? sO : sE, eg0,
               [&](int pos, const uint32_t* row, uint32_t live, const uint4* lraw) {
                 Spinor<A> acc[NSL];
-                simd_hop_out<P, LS, true, RS>(acc, row, live, a.t, sO, NB, eg, w, lraw, ring, lane,
-                                          tid);
-                if (!a.trivial) {
-                  __syncthreads();   // the ring becomes the slice-exchange buffer
-                  dplus_slices<A, LS, NSL, true>(acc, buf, K, w, lane);
-                }
+                simd_hop_out<P, LS, RS>(acc, row, live, in, in_s, NB, eg, w, lraw, ring, lane,
+                                        tid, fs);
                 const long e = (long)pos * NB + eg;
+                if (on_o) {
+                  // P1: t = [D+ M5op^-1] Dh_oe (D+ p); P3: s = [M5op^-dag D+^dag] Dh_oe^dag y
+                  __syncthreads();   // the ring becomes the post buffer
 #pragma unroll
-                for (int j = 0; j < NSL; j++) {
-                  const int s = w + j * LSP;
+                  for (int j = 0; j < NSL; j++) to_buf(buf, acc[j], w + j * LSP, lane);
+                  __syncthreads();
+                  if (dag) post_recurrence<A, LS, true>(buf, K, tid, NT);
+                  else post_recurrence<A, LS, false>(buf, K, tid, NT);
+                  __syncthreads();
 #pragma unroll
-                  for (int q = 0; q < 12; q++) acc[j].c[q] = cscale(hs, acc[j].c[q]);
-                  add_m5<P, true>(acc[j], a.y, sE, e, s, LS, K);
-                  Spinor<A> rr;
-                  ld_spinor<P>(rr, a.r, sB, e, s);
-#pragma unroll
-                  for (int q = 0; q < 12; q++) {
-                    rr.c[q].x -= al * acc[j].c[q].x;
-                    rr.c[q].y -= al * acc[j].c[q].y;
+                  for (int j = 0; j < NSL; j++) {
+                    from_buf(acc[j], buf, w + j * LSP, lane);
+                    store_spinor<P>(a.t, sO, e, w + j * LSP, acc[j]);
                   }
-                  store_spinor<P>(a.r, sB, e, s, rr);
-                  round_to_storage<P>(rr);
-                  nrm += norm2(rr);
+                } else if (!dag) {
+                  // P2: y = M5op p - 1/4 Dh_eo t on E; <p, A_s p> = ||y||^2 over the block
+                  const A hs = A(-0.25);
+#pragma unroll
+                  for (int j = 0; j < NSL; j++) {
+                    const int s = w + j * LSP;
+#pragma unroll
+                    for (int q = 0; q < 12; q++) acc[j].c[q] = cscale(hs, acc[j].c[q]);
+                    if (pos < a.nBE) add_m5<P, false>(acc[j], a.p, sB, e, s, LS, K);
+                    nrm += norm2(acc[j]);
+                    if (!last) store_spinor<P>(a.y, sE, e, s, acc[j]);
+                  }
+                } else {
+                  // P4: r -= alpha (M5op^dag y - 1/4 D+^dag Dh_eo^dag s) on BE; ||r||^2
+                  const A hs = A(a.hs_b), al = alpha_s[lane];
+                  if (!a.trivial) {
+                    __syncthreads();   // the ring becomes the slice-exchange buffer
+                    dplus_slices<A, LS, NSL, true>(acc, buf, K, w, lane);
+                  }
+#pragma unroll
+                  for (int j = 0; j < NSL; j++) {
+                    const int s = w + j * LSP;
+#pragma unroll
+                    for (int q = 0; q < 12; q++) acc[j].c[q] = cscale(hs, acc[j].c[q]);
+                    add_m5<P, true>(acc[j], a.y, sE, e, s, LS, K);
+                    Spinor<A> rr;
+                    ld_spinor<P>(rr, a.r, sB, e, s);
+#pragma unroll
+                    for (int q = 0; q < 12; q++) {
+                      rr.c[q].x -= al * acc[j].c[q].x;
+                      rr.c[q].y -= al * acc[j].c[q].y;
+                    }
+                    store_spinor<P>(a.r, sB, e, s, rr);
+                    round_to_storage<P>(rr);
+                    nrm += norm2(rr);
+                  }
                 }
               });
-        write_partial<A, LSP>(nrm, red, part + ci * 32, w, lane);
+        if (!on_o) write_partial<A, LSP>(nrm, red, part + ci * 32, w, lane);
         if (!barrier()) return;
-        const double rr_new = slot_total(part, C, sc, w, lane);
-        beta = (rho > 0.0 && isfinite(rr_new)) ? rr_new / rho : 0.0;
-        rho = rr_new;
+        if (!on_o) {
+          const double tot = slot_total(part, C, sc, w, lane);
+          if (w == 0) {
+            const double rho = rho_s[lane];
+            if (!dag) {
+              alpha_s[lane] = A((tot > 0.0 && isfinite(tot)) ? rho / tot : 0.0);
+            } else {
+              beta_s[lane] = A((rho > 0.0 && isfinite(tot)) ? tot / rho : 0.0);
+              rho_s[lane] = tot;
+            }
+          }
+          __syncthreads();
+        }
       }
+      if (done) break;
       // ---- P5: x += alpha p, p = r + beta p, u = D+ p on BE
       {
-        const A al = A(alpha), be = A(beta);
+        const A al = alpha_s[lane], be = beta_s[lane];
         for (int pos = ci; pos < a.nBE; pos += C) {
           const long e = (long)pos * NB + eg;
           Spinor<A> pv[NSL];
