@@ -42,16 +42,17 @@
  * Requirements: X, Y, Z, T even and >= 2; Ls in {4, 6, 8, 10, 12, 16} (kernels are
  * specialised per Ls); the device must be sm_103 (GB300).
  *
- * Launch variants: every operator stage exists in a few compiled variants (register budget,
- * grid shape, how links and neighbours are staged, how the fifth-dimension post matrices are
- * applied).  Per process, the first launches of each (stage kind, lattice size) that carry no
- * solver stop flag cycle through them timed with CUDA events, and the fastest is kept.  All
- * variants agree bit for bit except the tensor-core and recurrence forms of the 16-bit post
- * and the packed-float2 FP32 form (another rounding order), each within its precision's
- * tolerance.  Environment switches: DWF_STAGE_VARIANT=<i> forces
- * variant i; DWF_TUNE_LOG=1 prints each decision on stderr; DWF_POST=matrix|recurrence and
- * DWF_DISABLE_TC=1 (read by dwf_create) restrict the post forms; DWF_RU_DELTA overrides the
- * reliable-update threshold 0.1 of the mixed-precision solvers.
+ * Launch variants: FP64 stages have one kernel whose launch shape follows from the sizes, FP32
+ * stages three variants chosen by size.  FP16/BF16 stages exist in a few compiled variants
+ * (register budget, grid shape, how links and neighbours are staged, how the fifth-dimension
+ * post matrices are applied): per process, the first launches of each (stage kind, lattice size)
+ * that carry no solver stop flag cycle through them timed with CUDA events, and the fastest is
+ * kept.  They agree bit for bit except the tensor-core and recurrence forms of the post (another
+ * rounding order), each within its precision's tolerance.  Environment switches:
+ * DWF_STAGE_VARIANT=<i> forces variant i of the FP32 and 16-bit stages; DWF_TUNE_LOG=1 prints
+ * each decision on stderr; DWF_POST=matrix|recurrence and DWF_DISABLE_TC=1 (read by dwf_create)
+ * restrict the post forms; DWF_RU_DELTA overrides the reliable-update threshold 0.1 of the
+ * mixed-precision solvers.
  */
 #ifndef DWF_H
 #define DWF_H

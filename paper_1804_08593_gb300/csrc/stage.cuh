@@ -17,7 +17,8 @@
 // over the CTA's 32 sites x 24 reals in shared memory: by bidiagonal recurrences, as a dense
 // column GEMM, or on the tensor cores.  The epilogue optionally fuses the CG residual update
 // r -= alpha * out and a deterministic ||.||^2 reduction.  Which variant runs is decided per
-// stage kind by the launch autotuner (stage_inst.cuh).
+// stage kind by size (FP32) or by the launch autotuner (FP16/BF16; stage_inst.cuh).  FP64 stages
+// have a kernel of their own (stage64.cuh).
 #pragma once
 
 #include "dwf_device.cuh"
@@ -164,27 +165,31 @@ __device__ __forceinline__ void hop_term16(Spinor<float>& acc, const uint4 (&q)[
   }
 }
 
-// How a stage gathers the eight neighbour spinors and its links (a launch-variant choice, timed
-// by the autotuner): neighbours straight into registers or through a two-slot cp.async ring in
+// How a stage gathers the eight neighbour spinors and its links (a launch-variant choice,
+// stage_inst.cuh): neighbours straight into registers or through a two-slot cp.async ring in
 // shared memory; links from global memory after an optional bulk L2 prefetch of the tile's
-// links (G_BPF_L; G_BPF_LS / G_RING_BPF also prefetch the streamed inputs: local-term input,
+// links (G_BPF_L; G_RING_BPF also prefetches the streamed inputs: local-term input,
 // residual), or copied into shared memory by the TMA engine (G_TMA / G_RING_TMA: one
 // cp.async.bulk per 512-byte run, completing on an mbarrier) and read by every warp from there.
 // Either way each tile's links come from DRAM once and no direction waits on DRAM for them.
-enum Gather { G_REG = 0, G_RING = 1, G_RING_BPF = 5, G_BPF_LS = 6, G_BPF_L = 7, G_TMA = 10,
+enum Gather { G_REG = 0, G_RING = 1, G_RING_BPF = 5, G_BPF_L = 7, G_TMA = 10,
               G_RING_TMA = 11 };
 __host__ __device__ constexpr bool gather_ring(int g) {
   return g == G_RING || g == G_RING_BPF || g == G_RING_TMA;
 }
 __host__ __device__ constexpr bool gather_tma(int g) { return g == G_TMA || g == G_RING_TMA; }
 // Slice mode of a stage launch: one fifth-dimension slice per thread, or two (slices w and
-// w + Ls/2, each link read once for both; FP32 with the links in shared memory), the latter
-// also with the two slices' components packed in float2 and f32x2 arithmetic.
-enum SliceMode { SP_ONE = 1, SP_PAIR = 2, SP_PAIR_F2 = 3 };
-__host__ __device__ constexpr int slices_per_thread(int sp) { return sp == SP_ONE ? 1 : 2; }
+// w + Ls/2, each link read once for both; FP32 with the links in shared memory).
+// SP_ONE_F2: one slice per thread with the two components of the projected half-spinor packed in
+// float2 (FP32): the SU(3) products and sums of one slice take half the instructions, without
+// the second slice's registers.
+enum SliceMode { SP_ONE = 1, SP_PAIR = 2, SP_ONE_F2 = 4 };
+__host__ __device__ constexpr int slices_per_thread(int sp) {
+  return sp == SP_PAIR ? 2 : 1;
+}
 // bulk-prefetch depth of a gather mode: 0 none, 1 links, 2 links and streamed inputs
 __host__ __device__ constexpr int bpf_what(int g) {
-  return g == G_BPF_LS ? 2 : g == G_BPF_L ? 1 : g == G_RING_BPF ? 2 : 0;
+  return g == G_BPF_L ? 1 : g == G_RING_BPF ? 2 : 0;
 }
 
 __device__ __forceinline__ void prefetch_l2_bulk(const void* p, uint32_t bytes) {
@@ -553,127 +558,108 @@ __device__ __forceinline__ void hop_pair(Spinor<typename Prec<P>::acc> (&acc)[2]
   hop_pair_d<P, 7, DAG, BLOCKED, COH>(acc, a, site, lane, w, lsp, lsm);
 }
 
-// Packed paired-slice hop (FP32): component k of slices w and w + lsp shares one float2, so
-// each f32x2 add or fma does the work of two FP32 instructions.  The projection to the
-// half-spinor is done per slice (its results pair up in registers); the SU(3) products, with
-// each link element broadcast to both halves, and the reconstruction run on the pairs.
+// Two values packed for f32x2 arithmetic, which does the work of two FP32 instructions: two
+// slices' (cx2, the local solver) or the two half-spinor components' (HopS2).
 struct cx2 {
   float2 x, y;   // real parts of the two slices, imaginary parts
 };
 __device__ __forceinline__ float2 bcast2(float v) { return make_float2(v, v); }
 
+// One slice with its half-spinor components packed: up = (spin 0, spin 1); lo = the lower
+// spins fed by component 0 and by component 1, (spin 3, spin 2) while x and y are summed,
+// (spin 2, spin 3) for z and t (the halves change places once in between).
+struct HopS2 {
+  float2 ux[3], uy[3], lx[3], ly[3];
+};
+
 template <int MU>
-__device__ __forceinline__ void hop_term_f2(cx2 (&acc)[12], const Spinor<float>& psi0,
-                                            const Spinor<float>& psi1, const cx<float> (&u)[9],
-                                            float sgn) {
-  cx<float> h0[2][3], h1[2][3];
-  project_half<float, MU>(h0, psi0, sgn);
-  project_half<float, MU>(h1, psi1, sgn);
-  cx2 h[2][3];
+__device__ __forceinline__ void hop_term_s2(HopS2& acc, const Spinor<float>& psi,
+                                            const cx<float> (&u)[9], float sgn) {
+  cx<float> hh[2][3];
+  project_half<float, MU>(hh, psi, sgn);
+  float2 hx[3], hy[3];
 #pragma unroll
-  for (int i = 0; i < 2; i++)
-#pragma unroll
-    for (int b = 0; b < 3; b++)
-      h[i][b] = {make_float2(h0[i][b].x, h1[i][b].x), make_float2(h0[i][b].y, h1[i][b].y)};
+  for (int b = 0; b < 3; b++) {
+    hx[b] = make_float2(hh[0][b].x, hh[1][b].x);
+    hy[b] = make_float2(hh[0][b].y, hh[1][b].y);
+  }
   const float2 m1 = bcast2(-1.f);
-  cx2 g[2][3];
+  // sgn * B^dag: i for x; -1, 1 for y; i, -i for z; 1 for t (components 0, 1)
+  const float2 f = MU == 1 ? make_float2(-sgn, sgn)
+                 : MU == 2 ? make_float2(sgn, -sgn) : bcast2(sgn);
+  const float2 nf = make_float2(-f.x, -f.y);
 #pragma unroll
   for (int a = 0; a < 3; a++) {
     const float2 ux0 = bcast2(u[3 * a].x), uy0 = bcast2(u[3 * a].y);
     const float2 ux1 = bcast2(u[3 * a + 1].x), uy1 = bcast2(u[3 * a + 1].y);
     const float2 ux2 = bcast2(u[3 * a + 2].x), uy2 = bcast2(u[3 * a + 2].y);
-#pragma unroll
-    for (int i = 0; i < 2; i++) {
-      // re: sum u.x h.x - sum u.y h.y;  im: sum u.x h.y + sum u.y h.x
-      float2 re = __fmul2_rn(ux0, h[i][0].x);
-      re = __ffma2_rn(ux1, h[i][1].x, re);
-      re = __ffma2_rn(ux2, h[i][2].x, re);
-      float2 q = __fmul2_rn(uy0, h[i][0].y);
-      q = __ffma2_rn(uy1, h[i][1].y, q);
-      q = __ffma2_rn(uy2, h[i][2].y, q);
-      float2 im = __fmul2_rn(ux0, h[i][0].y);
-      im = __ffma2_rn(ux1, h[i][1].y, im);
-      im = __ffma2_rn(ux2, h[i][2].y, im);
-      im = __ffma2_rn(uy0, h[i][0].x, im);
-      im = __ffma2_rn(uy1, h[i][1].x, im);
-      im = __ffma2_rn(uy2, h[i][2].x, im);
-      g[i][a] = {__ffma2_rn(q, m1, re), im};
-    }
-  }
-  // acc += v (s > 0) or acc -= v (s < 0): multiplying by -1 is exact, so the fma rounds once
-  // like a subtraction
-  auto add = [&](float2& acc_, float2 v, bool neg) {
-    acc_ = neg ? __ffma2_rn(v, m1, acc_) : __fadd2_rn(acc_, v);
-  };
-  const bool sn = sgn < 0.f;
-#pragma unroll
-  for (int a = 0; a < 3; a++) {
-    add(acc[a].x, g[0][a].x, false);
-    add(acc[a].y, g[0][a].y, false);
-    add(acc[3 + a].x, g[1][a].x, false);
-    add(acc[3 + a].y, g[1][a].y, false);
-    // lower spins: sgn * B^dag g, B^dag as in hop_term_u (i z = (-z.y, z.x))
-    if constexpr (MU == 0) {          // l0 = i g1, l1 = i g0
-      add(acc[6 + a].x, g[1][a].y, !sn);
-      add(acc[6 + a].y, g[1][a].x, sn);
-      add(acc[9 + a].x, g[0][a].y, !sn);
-      add(acc[9 + a].y, g[0][a].x, sn);
-    } else if constexpr (MU == 1) {   // l0 = g1, l1 = -g0
-      add(acc[6 + a].x, g[1][a].x, sn);
-      add(acc[6 + a].y, g[1][a].y, sn);
-      add(acc[9 + a].x, g[0][a].x, !sn);
-      add(acc[9 + a].y, g[0][a].y, !sn);
-    } else if constexpr (MU == 2) {   // l0 = i g0, l1 = -i g1
-      add(acc[6 + a].x, g[0][a].y, !sn);
-      add(acc[6 + a].y, g[0][a].x, sn);
-      add(acc[9 + a].x, g[1][a].y, sn);
-      add(acc[9 + a].y, g[1][a].x, !sn);
-    } else {                          // l0 = g0, l1 = g1
-      add(acc[6 + a].x, g[0][a].x, sn);
-      add(acc[6 + a].y, g[0][a].y, sn);
-      add(acc[9 + a].x, g[1][a].x, sn);
-      add(acc[9 + a].y, g[1][a].y, sn);
+    float2 re = __fmul2_rn(ux0, hx[0]);
+    re = __ffma2_rn(ux1, hx[1], re);
+    re = __ffma2_rn(ux2, hx[2], re);
+    float2 q = __fmul2_rn(uy0, hy[0]);
+    q = __ffma2_rn(uy1, hy[1], q);
+    q = __ffma2_rn(uy2, hy[2], q);
+    float2 im = __fmul2_rn(ux0, hy[0]);
+    im = __ffma2_rn(ux1, hy[1], im);
+    im = __ffma2_rn(ux2, hy[2], im);
+    im = __ffma2_rn(uy0, hx[0], im);
+    im = __ffma2_rn(uy1, hx[1], im);
+    im = __ffma2_rn(uy2, hx[2], im);
+    re = __ffma2_rn(q, m1, re);
+    acc.ux[a] = __fadd2_rn(acc.ux[a], re);
+    acc.uy[a] = __fadd2_rn(acc.uy[a], im);
+    if constexpr (MU == 0 || MU == 2) {   // times i
+      acc.lx[a] = __ffma2_rn(im, nf, acc.lx[a]);
+      acc.ly[a] = __ffma2_rn(re, f, acc.ly[a]);
+    } else {
+      acc.lx[a] = __ffma2_rn(re, f, acc.lx[a]);
+      acc.ly[a] = __ffma2_rn(im, f, acc.ly[a]);
     }
   }
 }
 
-template <int D, bool DAG, bool BLOCKED>
-__device__ __forceinline__ void hop_pair_f2_d(cx2 (&acc)[12], const StageArgs& a, long site,
-                                              int lane, int w, int lsp, const uint4* lsm) {
+template <int D, bool DAG, bool BLOCKED, bool LSM>
+__device__ __forceinline__ void hop_s2_d(HopS2& acc, const StageArgs& a, long site, long lsite,
+                                         int s, const void* lsm) {
   const uint32_t nb = __ldg(a.nbr + (long)D * a.Vp + site);
   const void* src;
   long vs;
   if (!nbr_source<BLOCKED>(a, nb, src, vs)) return;
-  const long j = (long)(nb & NBR_IDX);
   constexpr bool back = (D & 1) != 0;
   constexpr float sgn = (back != DAG) ? 1.f : -1.f;
-  Spinor<float> psi0, psi1;
-  load_spinor<P32>(psi0, src, vs, j, w);
-  load_spinor<P32>(psi1, src, vs, j, w + lsp);
+  Spinor<float> psi;
+  load_spinor<P32>(psi, src, vs, (long)(nb & NBR_IDX), s);
   cx<float> u[9];
-  load_link9<P32, true>(u, lsm, 32, lane, D);
-  hop_term_f2<D / 2>(acc, psi0, psi1, u, sgn);
+  load_link9<P32, LSM>(u, LSM ? lsm : a.links, LSM ? 32 : a.Vp_link, lsite, D);
+  hop_term_s2<D / 2>(acc, psi, u, sgn);
 }
 
-template <bool DAG, bool BLOCKED>
-__device__ __forceinline__ void hop_pair_f2(Spinor<float> (&out)[2], const StageArgs& a,
-                                            long site, int lane, int w, int lsp,
-                                            const uint4* lsm) {
-  cx2 acc[12];
+template <bool DAG, bool BLOCKED, bool LSM>
+__device__ __forceinline__ void hop_s2(Spinor<float>& out, const StageArgs& a, long site,
+                                       long lsite, int s, const void* lsm) {
+  HopS2 h;
+  const float2 z = make_float2(0.f, 0.f);
 #pragma unroll
-  for (int k = 0; k < 12; k++) acc[k] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-  hop_pair_f2_d<0, DAG, BLOCKED>(acc, a, site, lane, w, lsp, lsm);
-  hop_pair_f2_d<1, DAG, BLOCKED>(acc, a, site, lane, w, lsp, lsm);
-  hop_pair_f2_d<2, DAG, BLOCKED>(acc, a, site, lane, w, lsp, lsm);
-  hop_pair_f2_d<3, DAG, BLOCKED>(acc, a, site, lane, w, lsp, lsm);
-  hop_pair_f2_d<4, DAG, BLOCKED>(acc, a, site, lane, w, lsp, lsm);
-  hop_pair_f2_d<5, DAG, BLOCKED>(acc, a, site, lane, w, lsp, lsm);
-  hop_pair_f2_d<6, DAG, BLOCKED>(acc, a, site, lane, w, lsp, lsm);
-  hop_pair_f2_d<7, DAG, BLOCKED>(acc, a, site, lane, w, lsp, lsm);
+  for (int k = 0; k < 3; k++) h.ux[k] = h.uy[k] = h.lx[k] = h.ly[k] = z;
+  hop_s2_d<0, DAG, BLOCKED, LSM>(h, a, site, lsite, s, lsm);
+  hop_s2_d<1, DAG, BLOCKED, LSM>(h, a, site, lsite, s, lsm);
+  hop_s2_d<2, DAG, BLOCKED, LSM>(h, a, site, lsite, s, lsm);
+  hop_s2_d<3, DAG, BLOCKED, LSM>(h, a, site, lsite, s, lsm);
 #pragma unroll
-  for (int k = 0; k < 12; k++) {
-    out[0].c[k] = {acc[k].x.x, acc[k].y.x};
-    out[1].c[k] = {acc[k].x.y, acc[k].y.y};
+  for (int k = 0; k < 3; k++) {
+    h.lx[k] = make_float2(h.lx[k].y, h.lx[k].x);
+    h.ly[k] = make_float2(h.ly[k].y, h.ly[k].x);
+  }
+  hop_s2_d<4, DAG, BLOCKED, LSM>(h, a, site, lsite, s, lsm);
+  hop_s2_d<5, DAG, BLOCKED, LSM>(h, a, site, lsite, s, lsm);
+  hop_s2_d<6, DAG, BLOCKED, LSM>(h, a, site, lsite, s, lsm);
+  hop_s2_d<7, DAG, BLOCKED, LSM>(h, a, site, lsite, s, lsm);
+#pragma unroll
+  for (int k = 0; k < 3; k++) {
+    out.c[k] = {h.ux[k].x, h.uy[k].x};
+    out.c[3 + k] = {h.ux[k].y, h.uy[k].y};
+    out.c[6 + k] = {h.lx[k].x, h.ly[k].x};
+    out.c[9 + k] = {h.lx[k].y, h.ly[k].y};
   }
 }
 
@@ -744,7 +730,12 @@ __device__ __forceinline__ bool stage_tile(const StageArgs& a, long tile,
     if (__syncthreads_or(!ok)) return false;
     lsm = reinterpret_cast<const uint4*>(lk);
   }
-  if constexpr (SP == SP_ONE) {
+  if constexpr (SP == SP_ONE_F2) {
+    static_assert(P == P32 && !gather_ring(G) && !COH, "packed components: FP32, direct loads");
+    if constexpr (bpf_what(G) > 0) prefetch_tile<P, LS, BLOCKED, bpf_what(G)>(a, tile);
+    constexpr bool LSM = gather_tma(G);
+    if (valid) hop_s2<DAG, BLOCKED, LSM>(acc[0], a, site, LSM ? (long)lane : site, w, lsm);
+  } else if constexpr (SP == SP_ONE) {
     const int s = w;
     if constexpr (gather_ring(G)) {
       if constexpr (G == G_RING_BPF) prefetch_tile<P, LS, BLOCKED, 2>(a, tile);
@@ -785,11 +776,7 @@ __device__ __forceinline__ bool stage_tile(const StageArgs& a, long tile,
   } else {
     // paired slices (FP32, links staged in shared memory): one link load serves both slices
     static_assert(gather_tma(G), "paired slices read the links from shared memory");
-    static_assert(SP != SP_PAIR_F2 || P == P32, "packed pairs are FP32 only");
-    if (valid) {
-      if constexpr (SP == SP_PAIR) hop_pair<P, DAG, BLOCKED, COH>(acc, a, site, lane, w, LSP, lsm);
-      if constexpr (SP == SP_PAIR_F2) hop_pair_f2<DAG, BLOCKED>(acc, a, site, lane, w, LSP, lsm);
-    }
+    if (valid) hop_pair<P, DAG, BLOCKED, COH>(acc, a, site, lane, w, LSP, lsm);
   }
 
   if constexpr (POST == 2 && (P == P16 || P == PB16) && SP == SP_ONE) {
@@ -953,9 +940,10 @@ __device__ __forceinline__ bool stage_tile(const StageArgs& a, long tile,
     for (int k = 0; k < 12; k++) acc_j.c[k] = cscale(hs, acc_j.c[k]);
 
     if (a.local_mode != LOC_NONE && valid) {
-      // M5op x at s = alpha x_s + beta (P- x_{s+1} + P+ x_{s-1});
-      // M5op^dag x at s = alpha x_s + beta (P+ x_{s+1} + P- x_{s-1});
-      // x_{Ls} = -mf x_0, x_{-1} = -mf x_{Ls-1}.
+      // M5op x at s = alpha x_s + beta (P- x_{s+1} + P+ x_{s-1}) (local mode LOC_M5, of Dh
+      // stages), M5op^dag x at s = alpha x_s + beta (P+ x_{s+1} + P- x_{s-1}) (LOC_M5DAG, of
+      // Dh^dag stages); x_{Ls} = -mf x_0, x_{-1} = -mf x_{Ls-1}.  Which half of each
+      // neighbouring slice is needed is known at compile time: the other is not loaded.
       Spinor<A> x0, xu, xd;
       load_spinor<P, COH>(x0, a.in2, a.Vp, site, s);
       load_spinor<P, COH>(xu, a.in2, a.Vp, site, s + 1 < LS ? s + 1 : 0);
@@ -964,7 +952,7 @@ __device__ __forceinline__ bool stage_tile(const StageArgs& a, long tile,
       const A fu = (s + 1 < LS) ? A(1) : -C.mf;
       const A fd = (s > 0) ? A(1) : -C.mf;
       const A la = C.la, lb = C.lb;
-      const bool dagm = (a.local_mode == LOC_M5DAG);
+      constexpr bool dagm = DAG;
   #pragma unroll
       for (int k = 0; k < 12; k++) {
         const bool plus = k < 6;

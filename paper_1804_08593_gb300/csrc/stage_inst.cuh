@@ -60,16 +60,15 @@ struct StageTune {
   bool pending = false;
 };
 
-// The variants timed per stage kind (the first is the default for launches that are never
-// timed).  FP32 gathers into registers, plain or after a bulk L2 prefetch of the tile's links
-// (and streamed inputs), or with the tile's links copied into shared memory by the TMA engine,
-// with one or two fifth-dimension slices per thread; a register budget for 3 CTAs per SM
-// spills, and the cp.async ring, per-direction L1 prefetch, prefetching the neighbour runs and
-// prefetching the next tile of a persistent CTA measured slower.  FP16/BF16 gather through the
-// L1-cached cp.async ring with a register budget for 2 or 3 CTAs per SM, with the tile's links
-// and streams prefetched into L2 or its links staged in shared memory by TMA, one CTA per tile
-// (persistent grids measured 10-35 % slower there; only the tensor-core post, whose set-up is
-// per CTA, has them).  FP32: one CTA per tile or a persistent grid.
+// The variants per stage kind (the first is the default for launches that are never timed).
+// FP32 gathers into registers, plain or after a bulk L2 prefetch of the tile's links, with the
+// half-spinor components packed, or two slices per thread with the tile's links copied into
+// shared memory by the TMA engine, chosen by size (stage_rule32); cp.async rings of two or three
+// slots, prefetching the streamed inputs, the unpacked one-slice form and packed slice pairs
+// measured slower.  FP16/BF16 are timed: they gather through the L1-cached cp.async ring with a
+// register budget for 2 or 3 CTAs per SM, with the tile's links and streams prefetched into L2
+// or its links staged in shared memory by TMA, one CTA per tile (persistent grids measured
+// 10-35 % slower there; only the tensor-core post, whose set-up is per CTA, has them).
 template <int P, int LS, bool DAG, bool BLK, int POST, int MINB, int G, int SP = 1>
 static void stage_cand(StageCand* c, int& n, int per_sm) {
   c[n++] = {stage_launch_v<P, LS, DAG, BLK, POST, MINB, G, SP>,
@@ -96,18 +95,24 @@ static void stage_cands(StageCand* c, int& n) {
     stage_cand<P, LS, DAG, BLK, POST, MB, G_RING_BPF>(c, n, 0);
     stage_cand<P, LS, DAG, BLK, POST, MB, G_RING_TMA>(c, n, 0);
   } else {
-    stage_cand<P, LS, DAG, BLK, POST, 2, G_BPF_L>(c, n, 0);
-    stage_cand<P, LS, DAG, BLK, POST, 2, G_REG>(c, n, 0);
-    stage_cand<P, LS, DAG, BLK, POST, 2, G_BPF_LS>(c, n, 0);
-    stage_cand<P, LS, DAG, BLK, POST, 2, G_TMA>(c, n, 0);
-    stage_cand<P, LS, DAG, BLK, POST, 2, G_TMA>(c, n, 2);
-    // two slices per thread, one link load for both (half the warps, twice the loads each)
-    stage_cand<P, LS, DAG, BLK, POST, 2, G_TMA, SP_PAIR>(c, n, 0);
+    stage_cand<P, LS, DAG, BLK, POST, 2, G_BPF_L, SP_ONE_F2>(c, n, 0);
     stage_cand<P, LS, DAG, BLK, POST, 2, G_TMA, SP_PAIR>(c, n, 2);
-    // the same with the pairs packed in float2 (f32x2 arithmetic)
-    stage_cand<P, LS, DAG, BLK, POST, 2, G_TMA, SP_PAIR_F2>(c, n, 0);
-    stage_cand<P, LS, DAG, BLK, POST, 2, G_TMA, SP_PAIR_F2>(c, n, 2);
+    stage_cand<P, LS, DAG, BLK, POST, 2, G_REG, SP_ONE_F2>(c, n, 0);
   }
+}
+
+// FP32: which of the three variants above runs, by size (no timing: a solver's launches carry a
+// stop flag and are never timed).  The L2-to-SM traffic of the neighbour spinors bounds them
+// (about 8 TB/s: neither half the instructions nor twice the loads in flight changes the large
+// sizes by 5 %), so the packed component form wins by its registers, except where a CTA of Ls
+// warps leaves a second one no room: Ls = 16 pairs the slices (16^4: 240 us for the four stages
+// of a CG step against 297; at Ls = 12 it is level within 3 % on one problem and 7 % behind in
+// batches).  Up to two tiles per SM the links' L2 prefetch only delays the loads (8^3x16 x 12:
+// 37.2 us for the four stages against 38.6; 12^4 x 12: 85.3 both).
+template <int LS>
+static int stage_rule32(long ntiles) {
+  if (LS == 16) return 1;
+  return ntiles <= 2 * sm_count() ? 2 : 0;
 }
 
 template <int P, int LS, bool DAG, bool BLK>
@@ -150,6 +155,12 @@ static cudaError_t stage_launch_one(const StageArgs& a, cudaStream_t st) {
     for (int k = 0; k < n; k++)
       if (gather_tma(c[k].gather)) return c[k].fn(b, c[k].smem, grid_of(c[k]), st);
     return cudaErrorNotSupported;
+  }
+  const char* force = getenv("DWF_STAGE_VARIANT");
+  const bool forced = force && force[0] >= '0' && force[0] < '0' + n && force[1] == 0;
+  if constexpr (P == P32) {
+    const int v = forced ? force[0] - '0' : n == 1 ? 0 : stage_rule32<LS>(b.ntiles);
+    return c[v].fn(b, c[v].smem, grid_of(c[v]), st);
   }
   // per (device, tile count, kind); handles on different host threads share it
   static std::mutex mu;
@@ -195,9 +206,8 @@ static cudaError_t stage_launch_one(const StageArgs& a, cudaStream_t st) {
       T.pending = false;
     }
   }
-  const char* force = getenv("DWF_STAGE_VARIANT");
   int v = T.chosen >= 0 ? T.chosen : 0;
-  if (force && force[0] >= '0' && force[0] < '0' + n && force[1] == 0) {
+  if (forced) {
     v = force[0] - '0';
   } else if (T.chosen < 0 && T.next < nl && !capturing && a.stop == nullptr) {
     // launches that may return early (a solver's stop flag) are never timed: a converged
