@@ -26,17 +26,21 @@ static cudaError_t set_smem_once(K kernel, std::atomic<uint64_t>& done, int byte
 template <int P, int LS>
 __global__ void __launch_bounds__(32 * LS) vec_kernel(const VecArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
+  if constexpr (P == P64) programmatic_start();
   vec_tile<P, LS>(a, blockIdx.x, gridDim.x, smem_raw);
 }
 
 template <int P, int LS>
 static cudaError_t vec_launch(const VecArgs& a, cudaStream_t st) {
   using A = typename Prec<P>::acc;
-  const int w = P == P64 ? 1 << stage64_shape(a.Vp, LS, sm_count(), 1).lst : 32;
+  const int w = P == P64 ? 1 << stage64_shape(a.Vp, LS, sm_count(), false).lst : 32;
   const size_t sm = a.do_u ? (size_t)LS * 24 * w * sizeof(A) : 0;
   static std::atomic<uint64_t> attr{0};
   cudaError_t e = set_smem_once(vec_kernel<P, LS>, attr, (int)(LS * 24 * 32 * sizeof(A)));
   if (e != cudaSuccess) return e;
+  if constexpr (P == P64)
+    return launch_programmatic(a.Vp / w <= sm_count(), vec_kernel<P, LS>,
+                               dim3((unsigned)(a.Vp / w)), dim3(w, LS), sm, st, a);
   vec_kernel<P, LS><<<dim3((unsigned)(a.Vp / w)), dim3(w, LS), sm, st>>>(a);
   return cudaGetLastError();
 }

@@ -244,6 +244,27 @@ inline int sm_count() {
   return n;
 }
 
+// Launches a kernel that begins with programmatic_start(): with `early`, its CTAs are already
+// placed when the kernel in front of it on the stream ends.  For grids of at most one CTA per SM
+// only (FP64 solvers on the smallest lattices are chains of 10 us kernels: CG on 4^4 x 8 20.3 ->
+// 18.9 ms); a larger grid is placed wherever the running one happens to leave room, which
+// undoes the even spread that the FP64 stages depend on (8^3x16 x 8: 59 us a stage became 90).
+template <typename... A>
+cudaError_t launch_programmatic(bool early, void (*k)(A...), dim3 grid, dim3 block, size_t smem,
+                                cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = early ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k, args...);
+}
+
 // Field sizes in bytes.
 inline size_t real_bytes(int prec) { return prec == P64 ? 8 : prec == P32 ? 4 : 2; }
 inline size_t field_bytes(const Geom& g, int prec) {

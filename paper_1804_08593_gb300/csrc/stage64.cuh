@@ -13,13 +13,13 @@
 //    host (4 instructions per element instead of 7), scalings by 1 are left out.  (Taking
 //    g_f + g_b and g_b - g_f from one FMA chain would save another 12 of 216 instructions per
 //    direction pair and 5 % of the time, but turns infinite inputs into NaNs.)
-//  * Work has to reach every quarter of every SM.  A CTA is 2^lst sites x Ls slices, x DS = 8
+//  * Work has to reach every quarter of every SM.  A CTA is 2^lst sites x Ls slices, x DS = 16
 //    groups of threads (direction and half-spinor component) on lattices too small to fill
 //    the chip with whole hops; lst and DS are chosen at launch (stage64_shape).
 //
 // Measured, us per launch (stage A; before: one CTA per 32 sites, every instruction above):
-// 4^4 x 8 65 -> 11, 8^3x16 x 8 73 -> 58, 12^4 x 12 282 -> 220, 16^4 x 16 1019 -> 850 (94 % of
-// the FP64 rate on the instructions left), 16^3x32 x 12 1499 -> 1275.
+// 4^4 x 8 65 -> 8, 8^3x16 x 8 73 -> 56, 12^4 x 12 282 -> 212, 16^4 x 16 1019 -> 850 (94 % of the
+// FP64 rate on the instructions left), 16^3x32 x 12 1499 -> 1275.
 #pragma once
 
 #include "stage.cuh"
@@ -30,106 +30,117 @@ __device__ __forceinline__ double2 sel_swap(double2 v, bool swap) {
   return swap ? make_double2(v.y, v.x) : v;
 }
 
-// The hop in the directions +mu and -mu at one site and slice, for NI of the two components i
-// of the projected half-spinors, i0 .. i0 + NI - 1 (they are independent of each other).
-// up[n] += g_f + g_b goes to spin i, lo[n] += B^dag (g_b - g_f) (its lower partner) to spin
-// 2 + i, or 3 - i for x and y.  qf, qb: the slice's first chunk of the neighbour in the two
-// directions, site stride vf, vb (the blocked operators' halo neighbours live in another
-// array); has: the neighbour takes part; L: the link of direction 2 mu at this site, chunk
-// stride vl.
-template <bool DAG, int NI>
-__device__ __forceinline__ void hop64_pair(cx<double> (&up)[NI][3], cx<double> (&lo)[NI][3],
-                                           int mu, int i0, const double2* qf, long vf,
-                                           bool has_f, const double2* qb, long vb, bool has_b,
-                                           const double2* L, long vl) {
-  // (1 + sg gamma_mu) = [[1, sg B], [sg B^dag, 1]]; (B psi_dn)_i takes spin 3 - i (x and y) or
-  // 2 + i (z and t) with real and imaginary part swapped for x and z, times the signs m; B^dag
-  // swaps alike, times the signs n
-  const bool im = (mu & 1) == 0;
-  double mx[NI], my[NI], nx[NI], ny[NI];
-  int kp[NI];   // first component of the partner spin
+// Component i of the projected half-spinor in direction mu: (1 + sg gamma_mu) =
+// [[1, sg B], [sg B^dag, 1]]; (B psi_dn)_i takes spin 3 - i (x and y) or 2 + i (z and t), whose
+// first component is kp, with real and imaginary part swapped for x and z, times the signs m.
+// B^dag feeds the product g_i to spin 2 (`two`) or 3, swapped alike, times the signs n.
+struct HalfSpin {
+  int kp;
+  bool swap, two;
+  double mx, my, nx, ny;
+};
+__device__ __forceinline__ HalfSpin half_spin(int mu, int i) {
+  HalfSpin h;
+  h.swap = (mu & 1) == 0;
+  h.kp = mu < 2 ? 9 - 3 * i : 6 + 3 * i;
+  h.mx = i == 0 ? (mu == 1 ? -1.0 : 1.0) : (mu == 2 ? -1.0 : 1.0);
+  h.my = i == 0 ? (mu == 3 ? 1.0 : -1.0) : (mu == 0 ? -1.0 : 1.0);
+  h.two = (mu < 2) == (i == 1);
+  h.nx = h.two ? (h.swap ? -1.0 : 1.0) : (mu < 2 ? -1.0 : 1.0);
+  h.ny = h.two ? 1.0 : ((mu == 1 || mu == 2) ? -1.0 : 1.0);
+  return h;
+}
+
+// h = the projected component of the neighbour at q (site stride v), sg the sign of gamma; zero
+// where the neighbour is absent.
+__device__ __forceinline__ void project64(cx<double> (&h)[3], const HalfSpin& f, int i,
+                                          const double2* q, long v, bool has, double sg) {
 #pragma unroll
-  for (int n = 0; n < NI; n++) {
-    const int i = i0 + n;
-    kp[n] = mu < 2 ? 9 - 3 * i : 6 + 3 * i;
-    mx[n] = i == 0 ? (mu == 1 ? -1.0 : 1.0) : (mu == 2 ? -1.0 : 1.0);
-    my[n] = i == 0 ? (mu == 3 ? 1.0 : -1.0) : (mu == 0 ? -1.0 : 1.0);
-    // signs of the lower spin this component feeds: spin 2 for (mu >= 2, i = 0) and
-    // (mu < 2, i = 1), else spin 3
-    const bool two = (mu < 2) == (i == 1);
-    nx[n] = two ? (im ? -1.0 : 1.0) : (mu < 2 ? -1.0 : 1.0);
-    ny[n] = two ? 1.0 : ((mu == 1 || mu == 2) ? -1.0 : 1.0);
+  for (int a = 0; a < 3; a++) {
+    h[a] = {0.0, 0.0};
+    if (has) {
+      const double2 p = __ldg(q + (3 * i + a) * v);
+      const double2 b = sel_swap(__ldg(q + (f.kp + a) * v), f.swap);
+      h[a] = {fma(sg * f.mx, b.x, p.x), fma(sg * f.my, b.y, p.y)};
+    }
   }
+}
+
+// The hop in the directions +mu and -mu at one site and slice for both components:
+// up[i] += g_f + g_b (spin i), lo[i] += B^dag (g_b - g_f) (spin 3 - i for x and y, 2 + i for z
+// and t).  qf, qb: the slice's first chunk of the neighbour in the two directions, site stride
+// vf, vb (the blocked operators' halo neighbours live in another array); has: the neighbour
+// takes part; L: the link of direction 2 mu at this site, chunk stride vl.
+template <bool DAG>
+__device__ __forceinline__ void hop64_pair(cx<double> (&up)[2][3], cx<double> (&lo)[2][3],
+                                           int mu, const double2* qf, long vf, bool has_f,
+                                           const double2* qb, long vb, bool has_b,
+                                           const double2* L, long vl) {
+  const HalfSpin f[2] = {half_spin(mu, 0), half_spin(mu, 1)};
   constexpr double F = DAG ? 1.0 : -1.0;   // sign of gamma in the forward hop
-  auto project = [&](cx<double> (&h)[NI][3], const double2* q, long v, bool has, double sg) {
+  cx<double> h[2][3], gf[2][3];
 #pragma unroll
-    for (int n = 0; n < NI; n++)
-#pragma unroll
-      for (int a = 0; a < 3; a++) {
-        h[n][a] = {0.0, 0.0};
-        if (has) {
-          const double2 p = __ldg(q + (3 * (i0 + n) + a) * v);
-          const double2 b = sel_swap(__ldg(q + (kp[n] + a) * v), im);
-          h[n][a] = {fma(sg * mx[n], b.x, p.x), fma(sg * my[n], b.y, p.y)};
-        }
-      }
-  };
-  cx<double> h[NI][3], gf[NI][3];
-  project(h, qf, vf, has_f, F);
+  for (int n = 0; n < 2; n++) project64(h[n], f[n], n, qf, vf, has_f, F);
 #pragma unroll
   for (int a = 0; a < 3; a++) {
 #pragma unroll
-    for (int n = 0; n < NI; n++) gf[n][a] = {0.0, 0.0};
+    for (int n = 0; n < 2; n++) gf[n][a] = {0.0, 0.0};
 #pragma unroll
     for (int b = 0; b < 3; b++) {
       const double2 u = __ldg(L + (a * 3 + b) * vl);
 #pragma unroll
-      for (int n = 0; n < NI; n++) cfma(gf[n][a], cx<double>{u.x, u.y}, h[n][b]);
+      for (int n = 0; n < 2; n++) cfma(gf[n][a], cx<double>{u.x, u.y}, h[n][b]);
     }
   }
-  project(h, qb, vb, has_b, -F);
+#pragma unroll
+  for (int n = 0; n < 2; n++) project64(h[n], f[n], n, qb, vb, has_b, -F);
   L += 9 * vl;
   constexpr double G = DAG ? -1.0 : 1.0;   // lower spins: B^dag D, D = g_b - g_f (DAG: -D)
 #pragma unroll
   for (int a = 0; a < 3; a++) {
-    cx<double> gb[NI];
+    cx<double> gb[2];
 #pragma unroll
-    for (int n = 0; n < NI; n++) gb[n] = {0.0, 0.0};
+    for (int n = 0; n < 2; n++) gb[n] = {0.0, 0.0};
 #pragma unroll
     for (int b = 0; b < 3; b++) {
       const double2 u = __ldg(L + (a * 3 + b) * vl);
 #pragma unroll
-      for (int n = 0; n < NI; n++) cfma(gb[n], cx<double>{u.x, u.y}, h[n][b]);
+      for (int n = 0; n < 2; n++) cfma(gb[n], cx<double>{u.x, u.y}, h[n][b]);
     }
 #pragma unroll
-    for (int n = 0; n < NI; n++) {
+    for (int n = 0; n < 2; n++) {
       up[n][a] = cadd(up[n][a], cadd(gf[n][a], gb[n]));
       const cx<double> d = csub(gb[n], gf[n][a]);
-      const double2 l = sel_swap(make_double2(d.x, d.y), im);
-      lo[n][a].x = fma(G * nx[n], l.x, lo[n][a].x);
-      lo[n][a].y = fma(G * ny[n], l.y, lo[n][a].y);
+      const double2 l = sel_swap(make_double2(d.x, d.y), f[n].swap);
+      lo[n][a].x = fma(G * f[n].nx, l.x, lo[n][a].x);
+      lo[n][a].y = fma(G * f[n].ny, l.y, lo[n][a].y);
     }
   }
 }
 
 // Threads: site (tid mod 2^lst), slice, group (direction, half-spinor component);
-// LS * 2^lst * DS is a multiple of 32 and at most STAGE64_THREADS.
-constexpr int STAGE64_THREADS = 192;
+// LS * 2^lst * DS is a multiple of 32 and at most stage64_threads(DS).
+__host__ __device__ constexpr int stage64_threads(int ds) { return ds == 1 ? 192 : 256; }
+constexpr int STAGE64_DS = 16;   // direction groups where a site and slice is split
 
-// Shared memory: the hop results, [24 reals][LS][st], per direction with direction groups, and
-// for the dense post its matrices.
+// Shared memory: the results, [24 reals][LS][st], or the half-spinor products of the direction
+// groups, [16][6 reals][LS][st] (then the results); for the dense post its matrices.
+__host__ __device__ constexpr int stage64_hop_doubles(int ds) { return ds > 1 ? 96 : 24; }
 inline size_t stage64_smem(int Ls, int post, int st, int ds) {
   size_t b = 0;
-  if (post || ds > 1) b = (size_t)(ds > 1 ? 4 : 1) * 24 * Ls * st * sizeof(double);
+  if (post || ds > 1) b = (size_t)stage64_hop_doubles(ds) * Ls * st * sizeof(double);
   if (post == 1) b += (size_t)2 * Ls * Ls * sizeof(double);
   return b;
 }
 
+// Whole hops: two CTAs' worth of registers (168 a thread) keep three warps per SM quarter
+// resident (12^4 x 12: 974 us a CG iteration; with the 186 that the compiler takes freely 1034).
 template <int LS, bool DAG, bool BLOCKED, int POST, int DS>
-__global__ void __launch_bounds__(STAGE64_THREADS) stage64_kernel(const StageArgs a,
-                                                                  const int lst) {
+__global__ void __launch_bounds__(stage64_threads(DS), DS == 1 ? 2 : 1)
+    stage64_kernel(const StageArgs a, const int lst) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ double red_scratch[32];
+  programmatic_start();
   const int st = 1 << lst, tid = threadIdx.x, nt = blockDim.x;
   const long tile = blockIdx.x;
   const int sl = tid & (st - 1), rest = tid >> lst;
@@ -161,53 +172,48 @@ __global__ void __launch_bounds__(STAGE64_THREADS) stage64_kernel(const StageArg
   }
   const bool valid = jl < vh;
 
-  // up: spins 0, 1 (the one this thread computes); lo: spins 2, 3 (its lower partner)
-  constexpr int NI = DS == 1 ? 2 : 1;
-  cx<double> up[NI][3], lo[NI][3];
-#pragma unroll
-  for (int n = 0; n < NI; n++)
-#pragma unroll
-    for (int k = 0; k < 3; k++) up[n][k] = lo[n][k] = {0.0, 0.0};
-  const int i0 = DS == 1 ? 0 : dg >> 2, mu0 = DS == 1 ? 0 : dg & 3;
-#pragma unroll 1
-  for (int mu = mu0; mu < 4; mu += DS) {
-    if (DS == 1 && mu == 2) {   // x and y feed the lower spins crosswise, z and t straight
-#pragma unroll
-      for (int k = 0; k < 3; k++) {
-        const cx<double> t = lo[0][k];
-        lo[0][k] = lo[NI - 1][k];
-        lo[NI - 1][k] = t;
-      }
-    }
-    if (!valid) continue;
-    const void* src[2];
-    long vs[2], j[2];
-    bool has[2];
-#pragma unroll
-    for (int f = 0; f < 2; f++) {
-      const uint32_t nb = __ldg(a.nbr + (long)(2 * mu + f) * a.Vp + site);
-      has[f] = nbr_source<BLOCKED>(a, nb, src[f], vs[f]);
-      j[f] = (long)(nb & NBR_IDX);
-    }
-    if (BLOCKED && !has[0] && !has[1]) continue;
-    hop64_pair<DAG, NI>(up, lo, mu, i0,
-                        reinterpret_cast<const double2*>(src[0]) + s * 12 * vs[0] + j[0], vs[0],
-                        has[0], reinterpret_cast<const double2*>(src[1]) + s * 12 * vs[1] + j[1],
-                        vs[1], has[1],
-                        reinterpret_cast<const double2*>(a.links) + (long)mu * 18 * a.Vp_link +
-                            site,
-                        a.Vp_link);
-  }
-
-  // this thread's share of the results: all 12 components, or (direction groups) the spin dg
-  // of the sum over the four directions, for the first four groups
-  constexpr int NC = DS == 1 ? 12 : 3;
-  const bool owner = DS == 1 || dg < 4;
+  // this thread's share of the results: all 12 components, or (direction groups) component dg,
+  // for the first twelve groups
+  constexpr int NC = DS == 1 ? 12 : 1;
+  const bool owner = DS == 1 || dg < 12;
   cx<double> v[NC];
-  double* buf = reinterpret_cast<double*>(smem_raw);   // [24][LS][st] (per direction)
+  double* buf = reinterpret_cast<double*>(smem_raw);
   const int vol = LS << lst;            // one real component of the CTA
   const int me = (s << lst) + sl;
   if constexpr (DS == 1) {
+    cx<double> up[2][3], lo[2][3];   // spins 0, 1 and their lower partners
+#pragma unroll
+    for (int n = 0; n < 2; n++)
+#pragma unroll
+      for (int k = 0; k < 3; k++) up[n][k] = lo[n][k] = {0.0, 0.0};
+#pragma unroll 1
+    for (int mu = 0; mu < 4; mu++) {
+      if (mu == 2) {   // x and y feed the lower spins crosswise, z and t straight
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+          const cx<double> t = lo[0][k];
+          lo[0][k] = lo[1][k];
+          lo[1][k] = t;
+        }
+      }
+      if (!valid) continue;
+      const void* src[2];
+      long vs[2], j[2];
+      bool has[2];
+#pragma unroll
+      for (int f = 0; f < 2; f++) {
+        const uint32_t nb = __ldg(a.nbr + (long)(2 * mu + f) * a.Vp + site);
+        has[f] = nbr_source<BLOCKED>(a, nb, src[f], vs[f]);
+        j[f] = (long)(nb & NBR_IDX);
+      }
+      if (BLOCKED && !has[0] && !has[1]) continue;
+      hop64_pair<DAG>(up, lo, mu, reinterpret_cast<const double2*>(src[0]) + s * 12 * vs[0] + j[0],
+                      vs[0], has[0],
+                      reinterpret_cast<const double2*>(src[1]) + s * 12 * vs[1] + j[1], vs[1],
+                      has[1],
+                      reinterpret_cast<const double2*>(a.links) + (long)mu * 18 * a.Vp_link + site,
+                      a.Vp_link);
+    }
 #pragma unroll
     for (int k = 0; k < 3; k++) {
       v[k] = up[0][k];
@@ -216,25 +222,56 @@ __global__ void __launch_bounds__(STAGE64_THREADS) stage64_kernel(const StageArg
       v[9 + k] = lo[1][k];
     }
   } else {
-    double* mine = buf + mu0 * 24 * vol + me;
-    const int kl = (mu0 < 2) == (i0 == 1) ? 6 : 9;   // the lower spin fed
+    // group dg: direction dg & 7, half-spinor component dg >> 3; its product g goes to shared
+    // memory, [direction][component][colour][re, im][vol]
+    const int d = dg & 7, i = dg >> 3, mu = d >> 1;
+    const double back = (d & 1) ? 1.0 : -1.0, sg = DAG ? -back : back;
+    cx<double> g[3] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}};
+    if (valid) {
+      const uint32_t nb = __ldg(a.nbr + (long)d * a.Vp + site);
+      const void* src;
+      long vs;
+      if (nbr_source<BLOCKED>(a, nb, src, vs)) {
+        cx<double> h[3];
+        project64(h, half_spin(mu, i), i,
+                  reinterpret_cast<const double2*>(src) + s * 12 * vs + (long)(nb & NBR_IDX), vs,
+                  true, sg);
+        const double2* L = reinterpret_cast<const double2*>(a.links) + (long)d * 9 * a.Vp_link +
+                           site;
 #pragma unroll
-    for (int k = 0; k < 3; k++) {
-      mine[2 * (3 * i0 + k) * vol] = up[0][k].x;
-      mine[(2 * (3 * i0 + k) + 1) * vol] = up[0][k].y;
-      mine[2 * (kl + k) * vol] = lo[0][k].x;
-      mine[(2 * (kl + k) + 1) * vol] = lo[0][k].y;
+        for (int c = 0; c < 3; c++)
+#pragma unroll
+          for (int b = 0; b < 3; b++) {
+            const double2 u = __ldg(L + (c * 3 + b) * a.Vp_link);
+            cfma(g[c], cx<double>{u.x, u.y}, h[b]);
+          }
+      }
+    }
+    double* mine = buf + (d * 2 + i) * 6 * vol + me;
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+      mine[2 * c * vol] = g[c].x;
+      mine[(2 * c + 1) * vol] = g[c].y;
     }
     __syncthreads();
+    v[0] = {0.0, 0.0};
     if (owner) {
+      const int sp = dg / 3, c = dg - 3 * sp;   // spin and colour of component dg
 #pragma unroll
-      for (int c = 0; c < NC; c++) {
-        const double* p = buf + 2 * (dg * NC + c) * vol + me;
-        v[c] = {p[0], p[vol]};
-#pragma unroll
-        for (int g = 1; g < 4; g++) {
-          v[c].x += p[g * 24 * vol];
-          v[c].y += p[g * 24 * vol + vol];
+      for (int e = 0; e < 8; e++) {
+        const int m = e >> 1;
+        if (sp < 2) {
+          const double* p = buf + ((e * 2 + sp) * 6 + 2 * c) * vol + me;
+          v[0].x += p[0];
+          v[0].y += p[vol];
+        } else {   // sg B^dag g of the component that feeds this spin
+          const int src_i = (m < 2) == (sp == 2) ? 1 : 0;
+          const HalfSpin f = half_spin(m, src_i);
+          const double se = ((e & 1) != 0) != DAG ? 1.0 : -1.0;
+          const double* p = buf + ((e * 2 + src_i) * 6 + 2 * c) * vol + me;
+          const double2 l = sel_swap(make_double2(p[0], p[vol]), f.swap);
+          v[0].x = fma(se * f.nx, l.x, v[0].x);
+          v[0].y = fma(se * f.ny, l.y, v[0].y);
         }
       }
     }
@@ -251,7 +288,7 @@ __global__ void __launch_bounds__(STAGE64_THREADS) stage64_kernel(const StageArg
       }
     }
     if constexpr (POST == 1) {
-      double* mat = buf + (DS == 1 ? 1 : 4) * 24 * vol;
+      double* mat = buf + stage64_hop_doubles(DS) * vol;
       const double* pm = reinterpret_cast<const double*>(post);
       for (int i = tid; i < 2 * LS * LS; i += nt) mat[i] = pm[i];
     }
@@ -308,7 +345,7 @@ __global__ void __launch_bounds__(STAGE64_THREADS) stage64_kernel(const StageArg
     }
   }
   if constexpr (POST == 1) {
-    const double* mat = buf + (DS == 1 ? 1 : 4) * 24 * vol;
+    const double* mat = buf + stage64_hop_doubles(DS) * vol;
     for (int col = tid; col < (24 << lst); col += nt) {
       const int c = col >> lst, l = col & (st - 1);
       const double* m = mat + (c >= 12 ? LS * LS : 0);
@@ -391,25 +428,24 @@ __global__ void __launch_bounds__(STAGE64_THREADS) stage64_kernel(const StageArg
 
 // The launch shape (sites per CTA 2^lst, direction groups ds) whose busiest SM quarter has the
 // least FP64 work: a quarter takes 64 cycles per warp-wide FP64 instruction, so its work is
-// its warps times their FP64 instructions, about 1000 with whole hops and 190 with a direction
+// its warps times their FP64 instructions, about 1000 with whole hops and 110 with a direction
 // and half-spinor component per thread.  Among equals the smaller CTA, whose warps spread more
 // evenly, unless a load would fetch less than 64 contiguous bytes.  Measured per stage launch:
 // 16^4 x 16, whole hops, 2 / 4 / 8 / 16 sites: 844 / 816 / 810 / 924 us; 8^3x16 x 8, 4 / 8 / 32
-// sites: 55 / 63 / 64 us, direction groups 62-68; 4^4 x 8, whole hops 35 us, direction groups
-// with 1 / 2 / 4 sites 11.2 / 10.8 / 11.7 us (one CTA of 32 sites x Ls before: 65 us).
+// sites: 55 / 63 / 64 us.
 struct Stage64Shape {
   int lst, ds;
 };
-inline Stage64Shape stage64_shape(long sites, int Ls, int nsm, int most_ds) {
+inline Stage64Shape stage64_shape(long sites, int Ls, int nsm, bool split) {
   Stage64Shape best{5, 1};
   double cost = -1.0;
-  for (int ds = 1; ds <= most_ds; ds += 7)
+  for (int ds = 1; ds <= (split ? STAGE64_DS : 1); ds += STAGE64_DS - 1)
     for (int lst = 5; lst >= 0; lst--) {
       const int threads = (Ls << lst) * ds;
-      if (threads % 32 != 0 || threads > STAGE64_THREADS) continue;
+      if (threads % 32 != 0 || threads > stage64_threads(ds)) continue;
       const int warps = threads / 32;
       const long per_sm = ((sites >> lst) + nsm - 1) / nsm;
-      double c = (double)((per_sm * warps + 3) / 4) * (ds == 1 ? 1000.0 : 190.0);
+      double c = (double)((per_sm * warps + 3) / 4) * (ds == 1 ? 1000.0 : 110.0);
       for (int w = warps; w > 1; w >>= 1) c *= 1.02;
       if (lst < 2) c *= 1.05;
       if (cost < 0.0 || c < cost) {

@@ -235,14 +235,15 @@ static cudaError_t stage64_launch(const StageArgs& a, int lst, cudaStream_t st) 
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
   }
-  k<<<dim3((unsigned)(a.ntiles * 32 >> lst)), dim3((unsigned)((LS << lst) * DS)), sm, st>>>(a, lst);
-  return cudaGetLastError();
+  const long ctas = a.ntiles * 32 >> lst;
+  return launch_programmatic(ctas <= sm_count(), k, dim3((unsigned)ctas),
+                             dim3((unsigned)((LS << lst) * DS)), sm, st, a, lst);
 }
 template <int LS, bool DAG, bool BLK, int POST>
 static cudaError_t stage64_launch_ds(const StageArgs& a, cudaStream_t st) {
-  const Stage64Shape s = stage64_shape(a.ntiles * 32, LS, sm_count(), 8);
-  return s.ds == 8 ? stage64_launch<LS, DAG, BLK, POST, 8>(a, s.lst, st)
-                   : stage64_launch<LS, DAG, BLK, POST, 1>(a, s.lst, st);
+  const Stage64Shape s = stage64_shape(a.ntiles * 32, LS, sm_count(), true);
+  return s.ds == 1 ? stage64_launch<LS, DAG, BLK, POST, 1>(a, s.lst, st)
+                   : stage64_launch<LS, DAG, BLK, POST, STAGE64_DS>(a, s.lst, st);
 }
 template <int LS, bool DAG, bool BLK>
 static cudaError_t stage64_launch_post(const StageArgs& a, cudaStream_t st) {
