@@ -116,11 +116,15 @@ static dwf_status read_doubles(dwf_ctx* h, const double* dev, int n, double* out
   return DWF_OK;
 }
 
-static dwf_status read_ints(dwf_ctx* h, const int* dev, int n, int* out) {
-  DWF_CUDA(cudaMemcpyAsync(h->h_pinned, dev, n * sizeof(int), cudaMemcpyDeviceToHost,
+// Integers and one double with one wait.
+static dwf_status read_flags(dwf_ctx* h, const int* dev, int n, int* out, const double* devd,
+                             double* outd) {
+  DWF_CUDA(cudaMemcpyAsync(h->h_pinned, devd, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+  DWF_CUDA(cudaMemcpyAsync(h->h_pinned + 1, dev, n * sizeof(int), cudaMemcpyDeviceToHost,
                            h->stream));
   DWF_CUDA(cudaStreamSynchronize(h->stream));
-  memcpy(out, h->h_pinned, n * sizeof(int));
+  *outd = h->h_pinned[0];
+  memcpy(out, h->h_pinned + 1, n * sizeof(int));
   return DWF_OK;
 }
 
@@ -212,6 +216,56 @@ static dwf_status cg_iteration(const OpEngine& E, const CGVectors& v, double* ds
   return vec(E, va);
 }
 
+// Eight CG iterations as a CUDA graph, replayed through the solve, for lattices whose kernels
+// are shorter than the host takes to launch them (about 10 us each with their arguments; 4^4 x 8:
+// 53 us an iteration launched one by one).  Every iteration of a solve has the same arguments,
+// but for the place in the caller's history after a restart (`same` false: launched directly).
+// Not while the profiler records events per launch, on the legacy stream, which cannot be
+// captured, or inside a caller's capture; the first iterations run directly.
+struct CgGraph {
+  static constexpr int N = 8;
+  static constexpr long MOST = 200000;   // sites x slices of one parity
+  cudaGraphExec_t exec = nullptr;
+  bool usable, warm = false;
+  explicit CgGraph(const OpEngine& E) {
+    const dwf_ctx* h = E.h;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    usable = E.g().Vp * h->Ls <= MOST && !h->prof.on && h->stream != nullptr &&
+             h->stream != cudaStreamLegacy && h->stream != cudaStreamPerThread &&
+             cudaStreamIsCapturing(h->stream, &cs) == cudaSuccess &&
+             cs == cudaStreamCaptureStatusNone;
+  }
+  ~CgGraph() {
+    if (exec) cudaGraphExecDestroy(exec);
+  }
+  template <typename F>
+  dwf_status iterations(dwf_ctx* h, int n, bool same, F one) {
+    if (usable && same && warm && n >= N && !exec) DWF_TRY(capture(h, one));
+    warm = true;
+    for (; exec && same && n >= N; n -= N) DWF_CUDA(cudaGraphLaunch(exec, h->stream));
+    for (; n > 0; n--) DWF_TRY(one());
+    return DWF_OK;
+  }
+  template <typename F>
+  dwf_status capture(dwf_ctx* h, F one) {
+    usable = false;   // once
+    if (cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeRelaxed) != cudaSuccess) {
+      cudaGetLastError();
+      return DWF_OK;
+    }
+    dwf_status st = DWF_OK;
+    for (int k = 0; k < N && st == DWF_OK; k++) st = one();
+    cudaGraph_t g = nullptr;
+    const cudaError_t e = cudaStreamEndCapture(h->stream, &g);
+    if (st == DWF_OK && e == cudaSuccess && g &&
+        cudaGraphInstantiate(&exec, g, 0) != cudaSuccess)
+      exec = nullptr;
+    cudaGetLastError();   // not capturable here: launched directly
+    if (g) cudaGraphDestroy(g);
+    return st;
+  }
+};
+
 static dwf_status run_cg(dwf_ctx* h, Layout* lay, const void* b_c128, void* x_c128, bool x0,
                          double tol, int maxit, int prec, dwf_stats* stats) {
   Timer timer;
@@ -281,6 +335,7 @@ static dwf_status run_cg(dwf_ctx* h, Layout* lay, const void* b_c128, void* x_c1
   // its residual grows by more than 1e6 (divergence); the last two restart p = r.
   const int cap = (prec == P16 || prec == PB16) ? 200 : (1 << 30);
   dwf_status status = DWF_OK;
+  CgGraph graph(E);
   while (true) {
     if (rr <= tol2) break;
     if (!std::isfinite(rr)) {
@@ -318,13 +373,12 @@ static dwf_status run_cg(dwf_ctx* h, Layout* lay, const void* b_c128, void* x_c1
     while (true) {
       const int n = std::min(chunk, maxit - iters - done_cycle);
       if (n <= 0) break;
-      for (int k = 0; k < n; k++)
-        DWF_TRY(cg_iteration(E, v, dsc, dfl, dhist ? dhist + total_hist : nullptr,
-                             dcurv ? dcurv + total_hist : nullptr,
-                             dhist ? hcap - total_hist : 0));
+      DWF_TRY(graph.iterations(h, n, !dhist || total_hist == 0, [&]() {
+        return cg_iteration(E, v, dsc, dfl, dhist ? dhist + total_hist : nullptr,
+                            dcurv ? dcurv + total_hist : nullptr, dhist ? hcap - total_hist : 0);
+      }));
       double rho;
-      DWF_TRY(read_ints(h, dfl, F_NFLAG, fl));
-      DWF_TRY(read_doubles(h, dsc + S_RHO, 1, &rho));
+      DWF_TRY(read_flags(h, dfl, F_NFLAG, fl, dsc + S_RHO, &rho));
       done_cycle = fl[F_ITER];
       if (!std::isfinite(rho)) {
         finite_cycle = false;

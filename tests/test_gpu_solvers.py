@@ -362,3 +362,27 @@ def test_cg_lanczos_kappa_matches_dense_spectrum():
     assert abs(lmax - ev[-1]) <= 1e-8 * ev[-1]
     assert abs(lmin - ev[0]) <= 1e-4 * ev[0]
     assert abs(kappa - ev[-1] / ev[0]) <= 1e-4 * kappa
+
+
+@pytest.mark.parametrize("prec,dims,Ls", [("f64", (4, 4, 4, 4), 8), ("f32", (4, 4, 4, 4), 8),
+                                          ("f64", (4, 6, 2, 6), 6)])
+@pytest.mark.parametrize("history", [0, 4000])
+def test_cg_on_its_own_stream_replays_the_same_iterations(prec, dims, Ls, history):
+    """A handle with a stream of its own replays CG iterations as a CUDA graph, one on the legacy
+    stream launches them one by one: the same kernels, so the same bits, also across restarts
+    (f32), with a history, and for maxit that ends inside a graph."""
+    import torch
+    dwf = lib()
+    rng = np.random.default_rng(29)
+    U = cuda(inputs.gauge_links(dims, 0.3, rng))
+    phi = cuda(inputs.even_source(dims, Ls, rng))
+    for maxit in (45, 5000):
+        got = []
+        for stream in (None, torch.cuda.Stream()):
+            h = dwf.dwf_create(dims, Ls, 1.8, 0.1, 1.5, 0.5, U, stream)
+            x = torch.zeros_like(phi)
+            torch.cuda.synchronize()
+            st = dwf.dwf_cg(h, phi, x, 1e-10, maxit, prec, history=history, raise_on_fail=False)
+            got.append((host(x), st["iterations"], st.get("history")))
+        assert got[0][1] == got[1][1] and got[0][2] == got[1][2]
+        assert np.array_equal(got[0][0], got[1][0])
