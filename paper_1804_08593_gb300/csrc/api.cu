@@ -73,15 +73,16 @@ dwf_status stage_buffer(dwf_ctx* h, const char* name, const void* user, size_t b
 dwf_status finish_output(dwf_ctx* h, void* user, const void* dev, size_t bytes) {
   if (dev != user)
     DWF_CUDA(cudaMemcpyAsync(user, dev, bytes, cudaMemcpyDeviceToHost, h->stream));
-  DWF_CUDA(cudaStreamSynchronize(h->stream));
   return check_device_error(h);
 }
 
+// Waits for the handle's stream; the error flag comes back through pinned memory on the same
+// wait (a copy to pageable memory waits by itself).
 dwf_status check_device_error(dwf_ctx* h) {
-  int e = 0;
-  DWF_CUDA(cudaMemcpyAsync(&e, h->dev_err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  int* e = reinterpret_cast<int*>(h->h_pinned);
+  DWF_CUDA(cudaMemcpyAsync(e, h->dev_err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
   DWF_CUDA(cudaStreamSynchronize(h->stream));
-  if (e) {
+  if (*e) {
     // a CTA that gave up left its reduction segment unfinished: clear the counters so the
     // handle's next reductions start from zero
     DWF_CUDA(cudaMemsetAsync(h->dev_err, 0, sizeof(int), h->stream));

@@ -449,14 +449,20 @@ __device__ __forceinline__ double to_double(float f) {
 // 192-byte spinors with consecutive threads on consecutive 16-byte components, the library's
 // side 512 bytes of one chunk.  Bound by HBM: 24^3x48 x 12 to FP32 0.335 -> 0.164 ms, back
 // 0.453 -> 0.182 ms (one thread per spinor before, 192 bytes apart, scaled in FP64).
-// The pitch of 13 keeps both directions free of bank conflicts.
+// The pitch of 13 keeps both directions free of bank conflicts.  A full field's two parities are
+// one launch (blockIdx.z).
 constexpr int PACK_THREADS = 128, PACK_PITCH = 13;
+struct PackFields {
+  void* f[2];
+  const int* map[2];
+};
 
 template <int P>
 __global__ void __launch_bounds__(PACK_THREADS)
-pack_field_kernel(const double2* __restrict__ src, void* dst, const int* __restrict__ map,
-                  long Vp, long nsrc) {
+pack_field_kernel(const double2* __restrict__ src, const PackFields a, long Vp, long nsrc) {
   constexpr int NCH = Prec<P>::NCH;
+  void* dst = blockIdx.z ? a.f[1] : a.f[0];
+  const int* __restrict__ map = blockIdx.z ? a.map[1] : a.map[0];
   __shared__ double2 sm[32 * PACK_PITCH];
   const long base = (long)blockIdx.x * 32;
   const int s = blockIdx.y, tid = threadIdx.x;
@@ -490,9 +496,10 @@ pack_field_kernel(const double2* __restrict__ src, void* dst, const int* __restr
 
 template <int P>
 __global__ void __launch_bounds__(PACK_THREADS)
-unpack_field_kernel(const void* src, double2* __restrict__ dst, const int* __restrict__ map,
-                    long Vp, long ndst) {
+unpack_field_kernel(const PackFields a, double2* __restrict__ dst, long Vp, long ndst) {
   constexpr int NCH = Prec<P>::NCH;
+  const void* src = blockIdx.z ? a.f[1] : a.f[0];
+  const int* __restrict__ map = blockIdx.z ? a.map[1] : a.map[0];
   __shared__ double2 sm[32 * PACK_PITCH];
   const long base = (long)blockIdx.x * 32;
   const int s = blockIdx.y, tid = threadIdx.x;
@@ -527,41 +534,37 @@ unpack_field_kernel(const void* src, double2* __restrict__ dst, const int* __res
 }
 
 // ---- launches ----
+// to_field: caller complex128 [Ls][nc][12] -> internal field (np parities), else back; through
+// the site maps (-1: a padding site, zero inside).
 template <int P>
-static void launch_pack_p(const void* src, void* dst, const int* map, long Vp, long nsrc, int Ls,
-                          cudaStream_t st) {
-  pack_field_kernel<P><<<dim3((unsigned)(Vp / 32), Ls), PACK_THREADS, 0, st>>>(
-      reinterpret_cast<const double2*>(src), dst, map, Vp, nsrc);
+static void move_fields_p(bool to_field, void* c128, const PackFields& f, int np, long Vp, long nc,
+                          int Ls, cudaStream_t st) {
+  const dim3 grid((unsigned)(Vp / 32), Ls, np);
+  double2* c = reinterpret_cast<double2*>(c128);
+  if (to_field) pack_field_kernel<P><<<grid, PACK_THREADS, 0, st>>>(c, f, Vp, nc);
+  else unpack_field_kernel<P><<<grid, PACK_THREADS, 0, st>>>(f, c, Vp, nc);
 }
-template <int P>
-static void launch_unpack_p(const void* src, void* dst, const int* map, long Vp, long ndst,
-                            int Ls, cudaStream_t st) {
-  unpack_field_kernel<P><<<dim3((unsigned)(Vp / 32), Ls), PACK_THREADS, 0, st>>>(
-      src, reinterpret_cast<double2*>(dst), map, Vp, ndst);
-}
-
-// Caller complex128 [Ls][nsrc][12] -> internal field and back, through the site map (-1: a
-// padding site, zero inside).
-cudaError_t launch_pack_field_to(int prec, const void* src, void* dst, const int* map, long Vp,
-                                 long nsrc, int Ls, cudaStream_t st) {
+static cudaError_t move_fields(bool to_field, int prec, void* c128, const PackFields& f, int np,
+                               long Vp, long nc, int Ls, cudaStream_t st) {
   switch (prec) {
-    case P64: launch_pack_p<P64>(src, dst, map, Vp, nsrc, Ls, st); break;
-    case P32: launch_pack_p<P32>(src, dst, map, Vp, nsrc, Ls, st); break;
-    case P16: launch_pack_p<P16>(src, dst, map, Vp, nsrc, Ls, st); break;
-    default: launch_pack_p<PB16>(src, dst, map, Vp, nsrc, Ls, st);
+    case P64: move_fields_p<P64>(to_field, c128, f, np, Vp, nc, Ls, st); break;
+    case P32: move_fields_p<P32>(to_field, c128, f, np, Vp, nc, Ls, st); break;
+    case P16: move_fields_p<P16>(to_field, c128, f, np, Vp, nc, Ls, st); break;
+    default: move_fields_p<PB16>(to_field, c128, f, np, Vp, nc, Ls, st);
   }
   return cudaGetLastError();
+}
+
+cudaError_t launch_pack_field_to(int prec, const void* src, void* dst, const int* map, long Vp,
+                                 long nsrc, int Ls, cudaStream_t st) {
+  return move_fields(true, prec, const_cast<void*>(src), {{dst, nullptr}, {map, nullptr}}, 1, Vp,
+                     nsrc, Ls, st);
 }
 
 cudaError_t launch_unpack_field_to(int prec, const void* src, void* dst, const int* map, long Vp,
                                    long ndst, int Ls, cudaStream_t st) {
-  switch (prec) {
-    case P64: launch_unpack_p<P64>(src, dst, map, Vp, ndst, Ls, st); break;
-    case P32: launch_unpack_p<P32>(src, dst, map, Vp, ndst, Ls, st); break;
-    case P16: launch_unpack_p<P16>(src, dst, map, Vp, ndst, Ls, st); break;
-    default: launch_unpack_p<PB16>(src, dst, map, Vp, ndst, Ls, st);
-  }
-  return cudaGetLastError();
+  return move_fields(false, prec, dst, {{const_cast<void*>(src), nullptr}, {map, nullptr}}, 1, Vp,
+                     ndst, Ls, st);
 }
 
 dwf_status pack_even(dwf_ctx* h, Layout* lay, const void* src_c128, void* dst, int prec) {
@@ -581,20 +584,18 @@ dwf_status unpack_even(dwf_ctx* h, Layout* lay, const void* src, int prec, void*
 dwf_status pack_full(dwf_ctx* h, Layout* lay, const void* src_c128, void* dst_even,
                      void* dst_odd, int prec) {
   const Geom& g = lay->g;
-  void* dst[2] = {dst_even, dst_odd};
-  for (int p = 0; p < 2; p++)
-    DWF_CUDA(launch_pack_field_to(prec, src_c128, dst[p], lay->lex[p], g.Vp, g.V, g.Ls,
-                                  h->stream));
+  DWF_CUDA(move_fields(true, prec, const_cast<void*>(src_c128),
+                       {{dst_even, dst_odd}, {lay->lex[0], lay->lex[1]}}, 2, g.Vp, g.V, g.Ls,
+                       h->stream));
   return DWF_OK;
 }
 
 dwf_status unpack_full(dwf_ctx* h, Layout* lay, const void* src_even, const void* src_odd,
                        int prec, void* dst_c128) {
   const Geom& g = lay->g;
-  const void* src[2] = {src_even, src_odd};
-  for (int p = 0; p < 2; p++)
-    DWF_CUDA(launch_unpack_field_to(prec, src[p], dst_c128, lay->lex[p], g.Vp, g.V, g.Ls,
-                                    h->stream));
+  DWF_CUDA(move_fields(false, prec, dst_c128,
+                       {{const_cast<void*>(src_even), const_cast<void*>(src_odd)},
+                        {lay->lex[0], lay->lex[1]}}, 2, g.Vp, g.V, g.Ls, h->stream));
   return DWF_OK;
 }
 
