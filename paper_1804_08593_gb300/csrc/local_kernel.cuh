@@ -229,8 +229,8 @@ __device__ __forceinline__ void hop_acc_out(const HopAcc<P>& h,
 // link element broadcast to both halves).  The sign of gamma is a runtime value, +-1 multiplied
 // inside the FMAs that add (the same roundings), so that Dh and Dh^dag share one copy of the
 // code: with four unrolled copies (one per hop phase, 150 KB) the kernel waited for
-// instructions (12^3x24, 32 blocks of 6^4, Ls = 12, l = 6: 1.63 ms a launch, now 1.40; 24^4,
-// 256 blocks: 7.21, now 7.19, where three CTAs per SM hide the rest).
+// instructions (12^3x24, 32 blocks of 6^4, Ls = 12, l = 6: 1.63 ms a launch, then 1.40; 24^4,
+// 256 blocks: 7.21, then 7.19, where three CTAs per SM hide the rest).
 template <int MU>
 __device__ __forceinline__ void hop_term_f2s(cx2 (&acc)[12], const Spinor<float>& psi0,
                                              const Spinor<float>& psi1, const cx<float> (&u)[9],
@@ -678,17 +678,29 @@ __device__ __forceinline__ void write_partial(A v, A (*red)[32], double* dst, in
   }
 }
 
-// Sum over the slot's C partials of this lane's block (fixed order); valid in every thread.
-__device__ __forceinline__ double slot_total(const double* part, int C, double* sc, int w,
+// Sum over the slot's C partials of this lane's block, valid in warp 0: every warp adds its
+// share in order, four loads in flight, then warp 0 the shares (a fixed order for a given C).
+// An FP64 addition takes 64 cycles of an SM quarter: one warp adding all 304 partials of a slot
+// that has the whole GPU took 10 us, twice an iteration (12^3x24, 32 blocks of 6^4, Ls = 12,
+// l = 6: 1.42 -> 1.22 ms a launch; 8^3x16, 4^4 blocks, Ls = 4: 0.66 -> 0.41 ms).
+template <int NW>
+__device__ __forceinline__ double slot_total(const double* part, int C, double (*sc)[32], int w,
                                              int lane) {
-  if (w == 0) {
-    double t = 0.0;
-    for (int c = 0; c < C; c++) t += __ldcg(part + c * 32 + lane);
-    sc[lane] = t;
+  double t = 0.0;
+  for (int c = w; c < C; c += 4 * NW) {
+    double v[4];
+#pragma unroll
+    for (int j = 0; j < 4; j++)
+      v[j] = c + j * NW < C ? __ldcg(part + (c + j * NW) * 32 + lane) : 0.0;
+#pragma unroll
+    for (int j = 0; j < 4; j++) t += v[j];
   }
+  sc[w][lane] = t;
   __syncthreads();
-  const double t = sc[lane];
-  __syncthreads();
+  if (w == 0) {
+#pragma unroll
+    for (int k = 1; k < NW; k++) t += sc[k][lane];
+  }
   return t;
 }
 
@@ -713,7 +725,7 @@ simd_local_kernel(const SimdArgs a) {
   uint4* ring = reinterpret_cast<uint4*>(region);   // during the hops
   A* buf = reinterpret_cast<A*>(region);            // afterwards
   __shared__ A red[LSP][32];
-  __shared__ double sc[32];
+  __shared__ double sc[LSP][32];
   // the CG scalars of the lanes' blocks, kept out of the registers that the hop needs
   __shared__ double rho_s[32];
   __shared__ A alpha_s[32], beta_s[32];
@@ -822,7 +834,7 @@ simd_local_kernel(const SimdArgs a) {
       }
       write_partial<A, LSP>(nrm, red, part + ci * 32, w, lane);
       if (!barrier()) return;
-      const double tot = slot_total(part, C, sc, w, lane);
+      const double tot = slot_total<LSP>(part, C, sc, w, lane);
       if (w == 0) rho_s[lane] = tot;
     }
     for (int k = 0; k < a.l; k++) {
@@ -921,7 +933,7 @@ simd_local_kernel(const SimdArgs a) {
         if (!on_o) write_partial<A, LSP>(nrm, red, part + ci * 32, w, lane);
         if (!barrier()) return;
         if (!on_o) {
-          const double tot = slot_total(part, C, sc, w, lane);
+          const double tot = slot_total<LSP>(part, C, sc, w, lane);
           if (w == 0) {
             const double rho = rho_s[lane];
             if (!dag) {
