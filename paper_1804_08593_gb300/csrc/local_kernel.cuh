@@ -230,7 +230,9 @@ __device__ __forceinline__ void hop_acc_out(const HopAcc<P>& h,
 // inside the FMAs that add (the same roundings), so that Dh and Dh^dag share one copy of the
 // code: with four unrolled copies (one per hop phase, 150 KB) the kernel waited for
 // instructions (12^3x24, 32 blocks of 6^4, Ls = 12, l = 6: 1.63 ms a launch, then 1.40; 24^4,
-// 256 blocks: 7.21, then 7.19, where three CTAs per SM hide the rest).
+// 256 blocks: 7.21, then 7.19, where three CTAs per SM hide the rest;
+// 6^4 blocks with Ls = 4, two warps a CTA: 0.77, then 0.95, the one shape that lost by it and
+// that slot_total's split brought back to 0.69).
 template <int MU>
 __device__ __forceinline__ void hop_term_f2s(cx2 (&acc)[12], const Spinor<float>& psi0,
                                              const Spinor<float>& psi1, const cx<float> (&u)[9],
