@@ -9,6 +9,7 @@
 namespace dwf {
 
 static thread_local std::string g_last_error = "no error";
+thread_local GraphRecorder* recording = nullptr;
 
 dwf_status set_error(dwf_status st, const std::string& msg) {
   g_last_error = msg;

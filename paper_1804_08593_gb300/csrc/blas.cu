@@ -38,11 +38,9 @@ static cudaError_t vec_launch(const VecArgs& a, cudaStream_t st) {
   static std::atomic<uint64_t> attr{0};
   cudaError_t e = set_smem_once(vec_kernel<P, LS>, attr, (int)(LS * 24 * 32 * sizeof(A)));
   if (e != cudaSuccess) return e;
-  if constexpr (P == P64)
-    return launch_programmatic(a.Vp / w <= sm_count(), vec_kernel<P, LS>,
-                               dim3((unsigned)(a.Vp / w)), dim3(w, LS), sm, st, a);
-  vec_kernel<P, LS><<<dim3((unsigned)(a.Vp / w)), dim3(w, LS), sm, st>>>(a);
-  return cudaGetLastError();
+  const bool early = P == P64 && a.Vp / w <= sm_count();
+  return launch_kernel(early, vec_kernel<P, LS>, dim3((unsigned)(a.Vp / w)), dim3(w, LS), sm, st,
+                       a);
 }
 
 template <int P>

@@ -79,7 +79,7 @@ template <typename A> struct Spinor {
   cx<A> c[12];  // index spin*3 + colour
 };
 
-// Programmatic dependent launch (launch_programmatic in dwf_internal.h): the CTAs of the next
+// Programmatic dependent launch (launch_kernel in dwf_internal.h): the CTAs of the next
 // kernel may be scheduled from here on; this kernel touches no memory before the one in front
 // of it has ended.
 __device__ __forceinline__ void programmatic_start() {

@@ -244,14 +244,48 @@ inline int sm_count() {
   return n;
 }
 
-// Launches a kernel that begins with programmatic_start(): with `early`, its CTAs are already
-// placed when the kernel in front of it on the stream ends.  For grids of at most one CTA per SM
+// Kernel launches recorded as the nodes of a graph, each after the one before it, while
+// `recording` of the host thread is set.  Added node by node instead of by stream capture: as
+// long as a stream is being captured, waiting for the device from any other host thread, and
+// for a blocking stream any use of the legacy stream, is refused and ends the capture too.
+struct GraphRecorder {
+  cudaGraph_t graph = nullptr;
+  cudaGraphNode_t last = nullptr;
+  cudaError_t add(const void* k, dim3 grid, dim3 block, size_t smem, void** args, bool early) {
+    cudaGraphNodeParams p{};
+    p.type = cudaGraphNodeTypeKernel;
+    p.kernel.func = const_cast<void*>(k);
+    p.kernel.gridDim = grid;
+    p.kernel.blockDim = block;
+    p.kernel.sharedMemBytes = (unsigned)smem;
+    p.kernel.kernelParams = args;   // copied by the call
+    cudaGraphEdgeData e{};
+    if (early) {
+      e.type = cudaGraphDependencyTypeProgrammatic;
+      e.from_port = cudaGraphKernelNodePortProgrammatic;
+    }
+    cudaGraphNode_t n = nullptr;
+    const cudaError_t r = cudaGraphAddNode(&n, graph, last ? &last : nullptr, last ? &e : nullptr,
+                                           last ? 1 : 0, &p);
+    if (r == cudaSuccess) last = n;
+    return r;
+  }
+};
+extern thread_local GraphRecorder* recording;
+
+// Launches a kernel, or adds it to the graph that the thread is recording.  `early`, for kernels
+// that begin with programmatic_start(): the CTAs are already placed when the kernel in front of
+// it on the stream ends.  For grids of at most one CTA per SM
 // only (FP64 solvers on the smallest lattices are chains of 10 us kernels: CG on 4^4 x 8 20.3 ->
 // 18.9 ms); a larger grid is placed wherever the running one happens to leave room, which
 // undoes the even spread that the FP64 stages depend on (8^3x16 x 8: 59 us a stage became 90).
 template <typename... A>
-cudaError_t launch_programmatic(bool early, void (*k)(A...), dim3 grid, dim3 block, size_t smem,
-                                cudaStream_t st, A... args) {
+cudaError_t launch_kernel(bool early, void (*k)(A...), dim3 grid, dim3 block, size_t smem,
+                          cudaStream_t st, A... args) {
+  if (recording) {
+    void* p[] = {const_cast<void*>(static_cast<const void*>(&args))...};
+    return recording->add(reinterpret_cast<const void*>(k), grid, block, smem, p, early);
+  }
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = block;

@@ -220,8 +220,8 @@ static dwf_status cg_iteration(const OpEngine& E, const CGVectors& v, double* ds
 // are shorter than the host takes to launch them (about 10 us each with their arguments; 4^4 x 8:
 // 53 us an iteration launched one by one).  Every iteration of a solve has the same arguments,
 // but for the place in the caller's history after a restart (`same` false: launched directly).
-// Not while the profiler records events per launch, on the legacy stream, which cannot be
-// captured, or inside a caller's capture; the first iterations run directly.
+// Not while the profiler records events per launch or inside a caller's capture; the first
+// iterations run directly.
 struct CgGraph {
   static constexpr int N = 8;
   static constexpr long MOST = 200000;   // sites x slices of one parity
@@ -230,8 +230,7 @@ struct CgGraph {
   explicit CgGraph(const OpEngine& E) {
     const dwf_ctx* h = E.h;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    usable = E.g().Vp * h->Ls <= MOST && !h->prof.on && h->stream != nullptr &&
-             h->stream != cudaStreamLegacy && h->stream != cudaStreamPerThread &&
+    usable = E.g().Vp * h->Ls <= MOST && !h->prof.on &&
              cudaStreamIsCapturing(h->stream, &cs) == cudaSuccess &&
              cs == cudaStreamCaptureStatusNone;
   }
@@ -240,29 +239,26 @@ struct CgGraph {
   }
   template <typename F>
   dwf_status iterations(dwf_ctx* h, int n, bool same, F one) {
-    if (usable && same && warm && n >= N && !exec) DWF_TRY(capture(h, one));
+    if (usable && same && warm && n >= N) record(one);
     warm = true;
     for (; exec && same && n >= N; n -= N) DWF_CUDA(cudaGraphLaunch(exec, h->stream));
     for (; n > 0; n--) DWF_TRY(one());
     return DWF_OK;
   }
+  // Nothing of the recorded iterations runs; if any of it fails they are launched directly.
   template <typename F>
-  dwf_status capture(dwf_ctx* h, F one) {
+  void record(F one) {
     usable = false;   // once
-    if (cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeRelaxed) != cudaSuccess) {
-      cudaGetLastError();
-      return DWF_OK;
-    }
-    dwf_status st = DWF_OK;
-    for (int k = 0; k < N && st == DWF_OK; k++) st = one();
-    cudaGraph_t g = nullptr;
-    const cudaError_t e = cudaStreamEndCapture(h->stream, &g);
-    if (st == DWF_OK && e == cudaSuccess && g &&
-        cudaGraphInstantiate(&exec, g, 0) != cudaSuccess)
+    GraphRecorder rec;
+    bool ok = cudaGraphCreate(&rec.graph, 0) == cudaSuccess;
+    recording = &rec;
+    for (int k = 0; k < N && ok; k++) ok = one() == DWF_OK;
+    recording = nullptr;
+    if (!ok || cudaGraphInstantiate(&exec, rec.graph, 0) != cudaSuccess) {
       exec = nullptr;
-    cudaGetLastError();   // not capturable here: launched directly
-    if (g) cudaGraphDestroy(g);
-    return st;
+      cudaGetLastError();
+    }
+    if (rec.graph) cudaGraphDestroy(rec.graph);
   }
 };
 

@@ -33,8 +33,8 @@ static cudaError_t stage_launch_v(const StageArgs& b, size_t sm, long g, cudaStr
     if (e != cudaSuccess) return e;
     attr_set.fetch_or(bit);
   }
-  k<<<dim3((unsigned)g), dim3(32, LS / slices_per_thread(SP)), sm, st>>>(b);
-  return cudaGetLastError();
+  return launch_kernel(false, k, dim3((unsigned)g), dim3(32, LS / slices_per_thread(SP)), sm, st,
+                       b);
 }
 
 // Online autotuner over the launch variants of one stage (register budget for 2 or 3
@@ -42,8 +42,8 @@ static cudaError_t stage_launch_v(const StageArgs& b, size_t sm, long g, cudaStr
 // launches of each (stage kind, problem size) cycle through the candidates bracketed by CUDA
 // events; once every candidate has been timed twice the fastest is used for good.  The timed
 // launches are the caller's real work, so tuning costs nothing extra.  Tuning happens outside
-// stream capture only (a captured launch uses the current choice), and only on launches
-// without a stop flag; until a kind is decided, other launches use the first candidate.
+// stream capture and graph recording (such a launch uses the current choice), and on launches
+// without a stop flag only; until a kind is decided, other launches use the first candidate.
 using StageFn = cudaError_t (*)(const StageArgs&, size_t, long, cudaStream_t);
 struct StageCand {
   StageFn fn;
@@ -171,7 +171,7 @@ static cudaError_t stage_launch_one(const StageArgs& a, cudaStream_t st) {
   const int nl = nt + n;                                    // tuning launches
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   cudaStreamIsCapturing(st, &cap);
-  const bool capturing = (cap != cudaStreamCaptureStatusNone);
+  const bool capturing = cap != cudaStreamCaptureStatusNone || recording;
   // event queries are not allowed while the stream is being captured: decide only outside
   if (!capturing && T.chosen < 0 && T.next >= nl && T.pending) {
     bool done = true;
@@ -236,8 +236,8 @@ static cudaError_t stage64_launch(const StageArgs& a, int lst, cudaStream_t st) 
     if (e != cudaSuccess) return e;
   }
   const long ctas = a.ntiles * 32 >> lst;
-  return launch_programmatic(ctas <= sm_count(), k, dim3((unsigned)ctas),
-                             dim3((unsigned)((LS << lst) * DS)), sm, st, a, lst);
+  return launch_kernel(ctas <= sm_count(), k, dim3((unsigned)ctas),
+                       dim3((unsigned)((LS << lst) * DS)), sm, st, a, lst);
 }
 template <int LS, bool DAG, bool BLK, int POST>
 static cudaError_t stage64_launch_ds(const StageArgs& a, cudaStream_t st) {
