@@ -217,16 +217,18 @@ static dwf_status cg_iteration(const OpEngine& E, const CGVectors& v, double* ds
 }
 
 // Eight CG iterations as a CUDA graph, replayed through the solve, for lattices whose kernels
-// are shorter than the host takes to launch them (about 10 us each with their arguments; 4^4 x 8:
-// 53 us an iteration launched one by one).  Every iteration of a solve has the same arguments,
-// but for the place in the caller's history after a restart (`same` false: launched directly).
-// Not while the profiler records events per launch or inside a caller's capture; the first
-// iterations run directly.
+// are shorter than the host takes to launch them (4^4 x 8, Shamir: 58 us an iteration launched one
+// by one, 45 replayed).  Every iteration of a solve has the same arguments, but for the place in
+// the caller's history after a restart (`same` false: launched directly).  Recording takes the
+// host about 150 us, which the second replay has earned back (24 iterations in all, f64 4^4 x 8:
+// 1.75 ms with a graph, 1.76 without; one replay only, 16 iterations: 1.30 and 1.15; 40: 2.69 and
+// 2.84; 120: 7.25 and 8.95): it waits for a chunk of two.  Not while the profiler records events
+// per launch or inside a caller's capture.
 struct CgGraph {
   static constexpr int N = 8;
   static constexpr long MOST = 200000;   // sites x slices of one parity
   cudaGraphExec_t exec = nullptr;
-  bool usable, warm = false;
+  bool usable;
   explicit CgGraph(const OpEngine& E) {
     const dwf_ctx* h = E.h;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -239,8 +241,7 @@ struct CgGraph {
   }
   template <typename F>
   dwf_status iterations(dwf_ctx* h, int n, bool same, F one) {
-    if (usable && same && warm && n >= N) record(one);
-    warm = true;
+    if (usable && same && n >= 2 * N) record(one);
     for (; exec && same && n >= N; n -= N) DWF_CUDA(cudaGraphLaunch(exec, h->stream));
     for (; n > 0; n--) DWF_TRY(one());
     return DWF_OK;
