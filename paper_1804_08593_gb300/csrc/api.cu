@@ -11,6 +11,48 @@ namespace dwf {
 static thread_local std::string g_last_error = "no error";
 thread_local GraphRecorder* recording = nullptr;
 
+cudaError_t GraphRecorder::kernel(const void* k, dim3 grid, dim3 block, size_t smem, void** args,
+                                  LaunchMode m) {
+  cudaGraphNodeParams p{};
+  p.type = cudaGraphNodeTypeKernel;
+  p.kernel.func = const_cast<void*>(k);
+  p.kernel.gridDim = grid;
+  p.kernel.blockDim = block;
+  p.kernel.sharedMemBytes = (unsigned)smem;
+  p.kernel.kernelParams = args;   // copied by the call
+  cudaGraphEdgeData e{};
+  if (m == LAUNCH_EARLY) {
+    e.type = cudaGraphDependencyTypeProgrammatic;
+    e.from_port = cudaGraphKernelNodePortProgrammatic;
+  }
+  cudaGraphNode_t n = nullptr;
+  cudaError_t r = cudaGraphAddNode(&n, graph, last ? &last : nullptr, last ? &e : nullptr,
+                                   last ? 1 : 0, &p);
+  if (r == cudaSuccess && m == LAUNCH_COOPERATIVE) {
+    cudaLaunchAttributeValue v{};
+    v.cooperative = 1;
+    r = cudaGraphKernelNodeSetAttribute(n, cudaLaunchAttributeCooperative, &v);
+  }
+  if (r == cudaSuccess) last = n;
+  return r;
+}
+
+cudaError_t GraphRecorder::clear(void* p, size_t bytes) {
+  cudaMemsetParams m{};
+  m.dst = p;
+  m.elementSize = 1;
+  m.width = bytes;
+  m.height = 1;
+  cudaGraphNode_t n = nullptr;
+  const cudaError_t r = cudaGraphAddMemsetNode(&n, graph, last ? &last : nullptr, last ? 1 : 0, &m);
+  if (r == cudaSuccess) last = n;
+  return r;
+}
+
+cudaError_t clear_async(void* p, size_t bytes, cudaStream_t st) {
+  return recording ? recording->clear(p, bytes) : cudaMemsetAsync(p, 0, bytes, st);
+}
+
 dwf_status set_error(dwf_status st, const std::string& msg) {
   g_last_error = msg;
   return st;

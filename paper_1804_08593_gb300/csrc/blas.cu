@@ -39,8 +39,8 @@ static cudaError_t vec_launch(const VecArgs& a, cudaStream_t st) {
   cudaError_t e = set_smem_once(vec_kernel<P, LS>, attr, (int)(LS * 24 * 32 * sizeof(A)));
   if (e != cudaSuccess) return e;
   const bool early = P == P64 && a.Vp / w <= sm_count();
-  return launch_kernel(early, vec_kernel<P, LS>, dim3((unsigned)(a.Vp / w)), dim3(w, LS), sm, st,
-                       a);
+  return launch_kernel(early ? LAUNCH_EARLY : LAUNCH_PLAIN, vec_kernel<P, LS>,
+                       dim3((unsigned)(a.Vp / w)), dim3(w, LS), sm, st, a);
 }
 
 template <int P>
@@ -170,8 +170,7 @@ static cudaError_t cast_go(const CastArgs& a, dim3 g, dim3 b, cudaStream_t st) {
   cudaError_t e = set_smem_once(cast_kernel<PI, PO>, attr, (int)(16 * 24 * 32 * sizeof(AO)));
   if (e != cudaSuccess) return e;
   const size_t sm = a.out3 ? (size_t)b.y * 24 * 32 * sizeof(AO) : 0;
-  cast_kernel<PI, PO><<<g, b, sm, st>>>(a);
-  return cudaGetLastError();
+  return launch_kernel(LAUNCH_PLAIN, cast_kernel<PI, PO>, g, b, sm, st, a);
 }
 
 template <int PI>
@@ -295,12 +294,11 @@ __global__ void vop_kernel(const VopArgs a) {
 template <int P>
 static cudaError_t vop_px(int px, const VopArgs& a, dim3 g, dim3 b, cudaStream_t st) {
   switch (px) {
-    case P64: vop_kernel<P, P64><<<g, b, 0, st>>>(a); break;
-    case P32: vop_kernel<P, P32><<<g, b, 0, st>>>(a); break;
-    case P16: vop_kernel<P, P16><<<g, b, 0, st>>>(a); break;
-    default: vop_kernel<P, PB16><<<g, b, 0, st>>>(a);
+    case P64: return launch_kernel(LAUNCH_PLAIN, vop_kernel<P, P64>, g, b, 0, st, a);
+    case P32: return launch_kernel(LAUNCH_PLAIN, vop_kernel<P, P32>, g, b, 0, st, a);
+    case P16: return launch_kernel(LAUNCH_PLAIN, vop_kernel<P, P16>, g, b, 0, st, a);
+    default: return launch_kernel(LAUNCH_PLAIN, vop_kernel<P, PB16>, g, b, 0, st, a);
   }
-  return cudaGetLastError();
 }
 
 cudaError_t launch_vop(int prec, int prec_x, const VopArgs& a, int Ls, cudaStream_t st) {

@@ -244,47 +244,58 @@ inline int sm_count() {
   return n;
 }
 
-// Kernel launches recorded as the nodes of a graph, each after the one before it, while
-// `recording` of the host thread is set.  Added node by node instead of by stream capture: as
-// long as a stream is being captured, waiting for the device from any other host thread, and
+// Kernel launches (and clears) recorded as the nodes of a graph, each after the one before it,
+// while `recording` of the host thread is set.  Added node by node instead of by stream capture:
+// as long as a stream is being captured, waiting for the device from any other host thread, and
 // for a blocking stream any use of the legacy stream, is refused and ends the capture too.
+enum LaunchMode { LAUNCH_PLAIN, LAUNCH_EARLY, LAUNCH_COOPERATIVE };
 struct GraphRecorder {
   cudaGraph_t graph = nullptr;
-  cudaGraphNode_t last = nullptr;
-  cudaError_t add(const void* k, dim3 grid, dim3 block, size_t smem, void** args, bool early) {
-    cudaGraphNodeParams p{};
-    p.type = cudaGraphNodeTypeKernel;
-    p.kernel.func = const_cast<void*>(k);
-    p.kernel.gridDim = grid;
-    p.kernel.blockDim = block;
-    p.kernel.sharedMemBytes = (unsigned)smem;
-    p.kernel.kernelParams = args;   // copied by the call
-    cudaGraphEdgeData e{};
-    if (early) {
-      e.type = cudaGraphDependencyTypeProgrammatic;
-      e.from_port = cudaGraphKernelNodePortProgrammatic;
-    }
-    cudaGraphNode_t n = nullptr;
-    const cudaError_t r = cudaGraphAddNode(&n, graph, last ? &last : nullptr, last ? &e : nullptr,
-                                           last ? 1 : 0, &p);
-    if (r == cudaSuccess) last = n;
-    return r;
-  }
+  cudaGraphNode_t last = nullptr;   // null: the next node starts a branch of its own
+  cudaError_t kernel(const void* k, dim3 grid, dim3 block, size_t smem, void** args, LaunchMode m);
+  cudaError_t clear(void* p, size_t bytes);
 };
 extern thread_local GraphRecorder* recording;
 
-// Launches a kernel, or adds it to the graph that the thread is recording.  `early`, for kernels
-// that begin with programmatic_start(): the CTAs are already placed when the kernel in front of
-// it on the stream ends.  For grids of at most one CTA per SM
+// An executable graph of recorded launches.
+struct RecordedGraph {
+  cudaGraphExec_t exec = nullptr;
+  ~RecordedGraph() {
+    if (exec) cudaGraphExecDestroy(exec);
+  }
+  // Records what issue(recorder) launches; false if any of it fails.  Nothing of it runs.
+  template <typename F>
+  bool record(F issue) {
+    GraphRecorder rec;
+    bool ok = cudaGraphCreate(&rec.graph, 0) == cudaSuccess;
+    if (ok) {
+      recording = &rec;
+      ok = issue(rec) == DWF_OK;
+      recording = nullptr;
+    }
+    ok = ok && cudaGraphInstantiate(&exec, rec.graph, 0) == cudaSuccess;
+    if (!ok) exec = nullptr;
+    if (rec.graph) cudaGraphDestroy(rec.graph);
+    cudaGetLastError();
+    return ok;
+  }
+};
+
+// Clears device memory in stream order, or records that.
+cudaError_t clear_async(void* p, size_t bytes, cudaStream_t st);
+
+// Launches a kernel, or records that.  LAUNCH_EARLY, for kernels that begin with
+// programmatic_start(): the CTAs are already placed when the kernel in front of it on the stream
+// ends.  For grids of at most one CTA per SM
 // only (FP64 solvers on the smallest lattices are chains of 10 us kernels: CG on 4^4 x 8 20.3 ->
 // 18.9 ms); a larger grid is placed wherever the running one happens to leave room, which
 // undoes the even spread that the FP64 stages depend on (8^3x16 x 8: 59 us a stage became 90).
 template <typename... A>
-cudaError_t launch_kernel(bool early, void (*k)(A...), dim3 grid, dim3 block, size_t smem,
+cudaError_t launch_kernel(LaunchMode m, void (*k)(A...), dim3 grid, dim3 block, size_t smem,
                           cudaStream_t st, A... args) {
   if (recording) {
     void* p[] = {const_cast<void*>(static_cast<const void*>(&args))...};
-    return recording->add(reinterpret_cast<const void*>(k), grid, block, smem, p, early);
+    return recording->kernel(reinterpret_cast<const void*>(k), grid, block, smem, p, m);
   }
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
@@ -292,10 +303,15 @@ cudaError_t launch_kernel(bool early, void (*k)(A...), dim3 grid, dim3 block, si
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  if (m == LAUNCH_EARLY) {
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+  } else {
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+  }
   cfg.attrs = attr;
-  cfg.numAttrs = early ? 1 : 0;
+  cfg.numAttrs = m == LAUNCH_PLAIN ? 0 : 1;
   return cudaLaunchKernelEx(&cfg, k, args...);
 }
 

@@ -284,8 +284,8 @@ static cudaError_t simd_launch(int prec, const SimdArgs& a, int Ls, int v, int* 
 // Launch-variant tuner of the local-solve kernel (FP32/FP16/BF16 have three variants: ring
 // depth and register budget): the first calls per precision run every variant once untimed,
 // then twice timed with CUDA events on the stream; once all events have completed (checked
-// without blocking at later calls) the fastest is kept.  Calls under stream capture use the
-// current choice.  DWF_LOCAL_VARIANT=<v> forces variant v.
+// without blocking at later calls) the fastest is kept.  Calls under stream capture or graph
+// recording use the current choice.  DWF_LOCAL_VARIANT=<v> forces variant v.
 constexpr int SIMD_NV = 3, SIMD_TUNE_ROUNDS = 4;
 
 bool simd_variant_decided(const SimdLocal* S, int prec) {
@@ -401,7 +401,8 @@ dwf_status simd_local_solve(dwf_ctx* h, SimdLocal* S, int prec, int l, const voi
   cudaStreamCaptureStatus capst = cudaStreamCaptureStatusNone;
   cudaStreamIsCapturing(h->stream, &capst);
   int timed = -1;
-  const int v = simd_pick(S, prec, h->stream, capst != cudaStreamCaptureStatusNone, &timed);
+  const int v = simd_pick(S, prec, h->stream,
+                          recording || capst != cudaStreamCaptureStatusNone, &timed);
   DWF_CUDA(simd_launch(prec, a, h->Ls, v, &cap, nsm, h->stream, true));
   if (cap < 1) return set_error(DWF_ERR_CUDA, "local-solve kernel cannot be resident");
   const int most = std::max(1, std::max(S->nE, S->nO) / 2);   // positions per CTA >= 2
@@ -421,7 +422,7 @@ dwf_status simd_local_solve(dwf_ctx* h, SimdLocal* S, int prec, int l, const voi
   }
   a.ctr = S->ctr;
   a.partial = S->partial;
-  DWF_CUDA(cudaMemsetAsync(S->ctr, 0, nslots * sizeof(unsigned), h->stream));
+  DWF_CUDA(clear_async(S->ctr, nslots * sizeof(unsigned), h->stream));
   const double R = (double)real_bytes(prec);
   // algorithmic bytes per local iteration: the four hop stages read their input once and
   // write their output once per site and slice, read the links of their sites once, plus the

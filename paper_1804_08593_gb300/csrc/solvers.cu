@@ -227,7 +227,7 @@ static dwf_status cg_iteration(const OpEngine& E, const CGVectors& v, double* ds
 struct CgGraph {
   static constexpr int N = 8;
   static constexpr long MOST = 200000;   // sites x slices of one parity
-  cudaGraphExec_t exec = nullptr;
+  RecordedGraph graph;
   bool usable;
   explicit CgGraph(const OpEngine& E) {
     const dwf_ctx* h = E.h;
@@ -236,30 +236,18 @@ struct CgGraph {
              cudaStreamIsCapturing(h->stream, &cs) == cudaSuccess &&
              cs == cudaStreamCaptureStatusNone;
   }
-  ~CgGraph() {
-    if (exec) cudaGraphExecDestroy(exec);
-  }
   template <typename F>
   dwf_status iterations(dwf_ctx* h, int n, bool same, F one) {
-    if (usable && same && n >= 2 * N) record(one);
-    for (; exec && same && n >= N; n -= N) DWF_CUDA(cudaGraphLaunch(exec, h->stream));
+    if (usable && same && n >= 2 * N) {
+      usable = false;   // once
+      graph.record([&](GraphRecorder&) -> dwf_status {
+        for (int k = 0; k < N; k++) DWF_TRY(one());
+        return DWF_OK;
+      });
+    }
+    for (; graph.exec && same && n >= N; n -= N) DWF_CUDA(cudaGraphLaunch(graph.exec, h->stream));
     for (; n > 0; n--) DWF_TRY(one());
     return DWF_OK;
-  }
-  // Nothing of the recorded iterations runs; if any of it fails they are launched directly.
-  template <typename F>
-  void record(F one) {
-    usable = false;   // once
-    GraphRecorder rec;
-    bool ok = cudaGraphCreate(&rec.graph, 0) == cudaSuccess;
-    recording = &rec;
-    for (int k = 0; k < N && ok; k++) ok = one() == DWF_OK;
-    recording = nullptr;
-    if (!ok || cudaGraphInstantiate(&exec, rec.graph, 0) != cudaSuccess) {
-      exec = nullptr;
-      cudaGetLastError();
-    }
-    if (rec.graph) cudaGraphDestroy(rec.graph);
   }
 };
 
@@ -494,26 +482,20 @@ static dwf_status precondition_stages(const OpEngine& Em, const OpEngine& Ei, co
                                       int l);
 
 // The preconditioner step of the persistent local solver (the local solves' launch and the
-// reductions that follow it) as a CUDA graph: captured once the solver's launch variant is
+// reductions that follow it) as a CUDA graph: recorded once the solver's launch variant is
 // decided (never while the per-launch profiler is on, whose events must be recorded per
 // launch), then replayed by every later preconditioner call of the solve.  Every argument of
 // the step (buffers, scalar slots, sizes) is the same on every call.  DWF_PRECOND_GRAPH=0
 // issues the launches directly.
 struct PcGraph {
-  cudaGraphExec_t exec = nullptr;
+  RecordedGraph graph;
   bool tried = false;
-  ~PcGraph() {
-    if (exec) cudaGraphExecDestroy(exec);
-  }
 };
 
 static bool pc_graph_enabled(dwf_ctx* h, const InnerVectors& iv) {
   const char* e = getenv("DWF_PRECOND_GRAPH");
   if (e && strcmp(e, "0") == 0) return false;
   if (h->prof.on || !iv.simd || !simd_variant_decided(iv.simd, iv.prec)) return false;
-  // the legacy default stream cannot be captured: handles created without a stream launch
-  // directly
-  if (h->stream == nullptr || h->stream == cudaStreamLegacy) return false;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   return cudaStreamIsCapturing(h->stream, &cs) == cudaSuccess &&
          cs == cudaStreamCaptureStatusNone;
@@ -563,39 +545,17 @@ static dwf_status precondition(const OpEngine& Em, const OpEngine& Ei, const voi
       DWF_TRY(cast(Em, ip, iv.xi, z, scaled ? nreal : 1.0, scaled ? dsc + S_RR : nullptr, 1,
                    r, Em.red(FIN_STORE, dsc + S_RZNEW), nullptr, zmap, zvp));
       DWF_TRY(vop(Em, VOP_DOT, rold, z, Em.red(FIN_STORE, dsc + S_TMP)));
-      pr_beta_kernel<<<1, 1, 0, Em.h->stream>>>(dsc);
-      DWF_CUDA(cudaGetLastError());
+      DWF_CUDA(launch_kernel(LAUNCH_PLAIN, pr_beta_kernel, dim3(1), dim3(1), 0, Em.h->stream,
+                             dsc));
     }
     return DWF_OK;
   };
-  cudaStream_t st = Em.h->stream;
-  if (pg && pg->exec) {
-    DWF_CUDA(cudaGraphLaunch(pg->exec, st));
-  } else if (pg && !pg->tried && pc_graph_enabled(Em.h, iv)) {
+  if (pg && !pg->tried && pc_graph_enabled(Em.h, iv)) {
     pg->tried = true;
-    if (cudaStreamBeginCapture(st, cudaStreamCaptureModeRelaxed) != cudaSuccess) {
-      cudaGetLastError();
-      return precondition(Em, Ei, r, z, iv, dsc, blk, nb, l, flexible, rold, zs, nullptr);
-    }
-    const dwf_status s_issue = issue();
-    cudaGraph_t graph = nullptr;
-    const cudaError_t e_end = cudaStreamEndCapture(st, &graph);
-    cudaError_t e_inst = cudaErrorUnknown;
-    if (s_issue == DWF_OK && e_end == cudaSuccess && graph)
-      e_inst = cudaGraphInstantiate(&pg->exec, graph, 0);
-    if (graph) cudaGraphDestroy(graph);
-    if (s_issue != DWF_OK) return s_issue;
-    if (e_end != cudaSuccess || e_inst != cudaSuccess) {
-      // not capturable here: nothing of the step ran, so issue it directly (and from now on)
-      cudaGetLastError();
-      pg->exec = nullptr;
-      DWF_TRY(issue());
-    } else {
-      DWF_CUDA(cudaGraphLaunch(pg->exec, st));
-    }
-  } else {
-    DWF_TRY(issue());
+    pg->graph.record([&](GraphRecorder&) { return issue(); });
   }
+  if (pg && pg->graph.exec) DWF_CUDA(cudaGraphLaunch(pg->graph.exec, Em.h->stream));
+  else DWF_TRY(issue());
   if (!flexible) {
     zs.src = iv.xi;
     zs.prec = ip;

@@ -33,8 +33,8 @@ static cudaError_t stage_launch_v(const StageArgs& b, size_t sm, long g, cudaStr
     if (e != cudaSuccess) return e;
     attr_set.fetch_or(bit);
   }
-  return launch_kernel(false, k, dim3((unsigned)g), dim3(32, LS / slices_per_thread(SP)), sm, st,
-                       b);
+  return launch_kernel(LAUNCH_PLAIN, k, dim3((unsigned)g), dim3(32, LS / slices_per_thread(SP)), sm,
+                       st, b);
 }
 
 // Online autotuner over the launch variants of one stage (register budget for 2 or 3
@@ -236,7 +236,7 @@ static cudaError_t stage64_launch(const StageArgs& a, int lst, cudaStream_t st) 
     if (e != cudaSuccess) return e;
   }
   const long ctas = a.ntiles * 32 >> lst;
-  return launch_kernel(ctas <= sm_count(), k, dim3((unsigned)ctas),
+  return launch_kernel(ctas <= sm_count() ? LAUNCH_EARLY : LAUNCH_PLAIN, k, dim3((unsigned)ctas),
                        dim3((unsigned)((LS << lst) * DS)), sm, st, a, lst);
 }
 template <int LS, bool DAG, bool BLK, int POST>

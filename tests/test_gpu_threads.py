@@ -74,3 +74,33 @@ def test_cg_beside_another_thread(prec, other, blocking):
     assert all(np.array_equal(g, alone) for g in got)
     h.close()
     free()
+
+
+@pytest.mark.parametrize("blocking", [False, True])
+@pytest.mark.parametrize("other", ["device_wait", "legacy_stream"])
+@pytest.mark.parametrize("flexible", [False, True])
+def test_mspcg_beside_another_thread(flexible, other, blocking):
+    import torch
+    dwf = lib()
+    dims, Ls = (8, 4, 4, 8), 8
+    rng = np.random.default_rng(37)
+    U, phi = cuda(inputs.gauge_links(dims, 0.2, rng)), cuda(inputs.even_source(dims, Ls, rng))
+    stream, free = _blocking_stream() if blocking else (torch.cuda.Stream(), lambda: None)
+    torch.cuda.synchronize()
+    h = dwf.dwf_create(dims, Ls, 1.8, 0.1, 1.5, 0.5, U, stream)
+
+    def solve():
+        x = torch.zeros_like(phi)
+        torch.cuda.current_stream().synchronize()
+        st = dwf.dwf_mspcg(h, (4, 4, 4, 4), 4, "f16", "f32", phi, x, 1e-10, 2000,
+                           local_op=dwf.LOCAL_EXACT, flexible=flexible)
+        assert st["true_residual"] <= 1e-10
+        return host(x)
+
+    for _ in range(4):     # the local solver's launch variant is decided
+        alone = solve()
+    got, errors = _beside(other, solve, 8)
+    assert not errors, errors
+    assert all(np.array_equal(g, alone) for g in got)
+    h.close()
+    free()
