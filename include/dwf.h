@@ -208,7 +208,7 @@ typedef struct {
  * group, either one persistent cooperative kernel launch (five phases per step separated by
  * grid barriers with bounded waits) or five launches per step (stages A, B, A^dag, B^dag on
  * persistent grids, then the update), whichever the first chunks time faster (the choice is
- * kept for later calls on the same problem mix); the chosen chunks of all groups are captured
+ * kept for later calls on the same problem mix); the chosen chunks of all groups are recorded
  * once as a CUDA graph and replayed, with the per-problem FP64 reliable updates between
  * replays.  stream: cudaStream_t.  per_solve (n entries,
  * nullable) receives each problem's statistics.  Fields are host or device; the call keeps

@@ -8,7 +8,7 @@
 // phases per step over all tiles, grid barriers with bounded waits) or five launches per step
 // (stages A, B, A^dag, B^dag on persistent grids, then the update); which one, the grid size
 // and the link staging are picked per group by timing the first chunks (and kept for later
-// calls on the same problem mix), and the chosen launches of all groups are then captured
+// calls on the same problem mix), and the chosen launches of all groups are then recorded
 // once in a CUDA graph and replayed.  FP32 CG with
 // FP64 reliable updates per problem (the true residual is recomputed in FP64 when a problem's
 // FP32 residual has dropped by delta = 0.1, or at convergence), between replays.
@@ -173,7 +173,6 @@ struct Batch {
   std::vector<std::unique_ptr<Group>> groups;
   cudaStream_t st = nullptr;
   bool own_stream = false;
-  std::vector<cudaStream_t> side;   // capture streams of the groups after the first
   double* staged_links = nullptr;
   unsigned long long wait_ns = 0;   // bounded device waits (DWF_WAIT_LIMIT_US; 0: default)
   std::vector<void*> owned;
@@ -181,7 +180,6 @@ struct Batch {
     if (st) cudaStreamSynchronize(st);
     groups.clear();
     for (void* p : owned) cudaFree(p);
-    for (cudaStream_t q : side) cudaStreamDestroy(q);
     if (own_stream) cudaStreamDestroy(st);
   }
 };
@@ -735,8 +733,7 @@ extern "C" dwf_status dwf_batch_solve(int n, const dwf_problem* problems, double
   if (!(tol > 0.0) || maxit < 0) return set_error(DWF_ERR_ARG, "bad tolerance or maxit");
   const auto t0 = std::chrono::steady_clock::now();
   Batch B;
-  // all work runs on a private non-blocking stream (stream capture is not possible on the
-  // legacy default stream), ordered after the caller's stream
+  // all work runs on a private non-blocking stream, ordered after the caller's stream
   cudaStream_t caller = reinterpret_cast<cudaStream_t>(stream);
   DWF_CUDA(cudaStreamCreateWithFlags(&B.st, cudaStreamNonBlocking));
   B.own_stream = true;
@@ -839,7 +836,7 @@ extern "C" dwf_status dwf_batch_solve(int n, const dwf_problem* problems, double
   // stage and update (g_cg_step, each stage with its own tuned variant).  The first chunks time
   // the candidates (the stage launches; the persistent launch with a grid of 1 or 2 CTAs per
   // SM or the largest co-resident grid, links read directly or staged by TMA bulk copies); the
-  // fastest of each group is then captured once in a CUDA graph and replayed.  Groups whose
+  // fastest of each group is then recorded once in a CUDA graph and replayed.  Groups whose
   // fifth-dimension post cannot use the recurrences keep the stage launches.
   const int chunk = 16;
   int dev = 0, nsm = 1;
@@ -895,95 +892,56 @@ extern "C" dwf_status dwf_batch_solve(int n, const dwf_problem* problems, double
   auto launch_chunk = [&](Group& G, int gather, int grid) -> dwf_status {
     BatchStepArgs ba;
     g_step_args(G, chunk, wait_ns, ba);
-    DWF_CUDA(cudaMemsetAsync(G.bar, 0, sizeof(unsigned), B.st));
+    DWF_CUDA(clear_async(G.bar, sizeof(unsigned), B.st));
     int cap = 0;
     DWF_CUDA(batch_steps_launch(ba, G.Ls, gather, grid, &cap, nsm, B.st, false));
     return DWF_OK;
   };
-  auto stage_chunk = [&](Group& G, cudaStream_t st) -> dwf_status {
-    for (int k = 0; k < chunk; k++) DWF_TRY(g_cg_step(G, st));
+  auto stage_chunk = [&](Group& G) -> dwf_status {
+    for (int k = 0; k < chunk; k++) DWF_TRY(g_cg_step(G, B.st));
     return DWF_OK;
   };
   size_t tune_round = 0;
-  cudaGraph_t graph = nullptr;
-  cudaGraphExec_t exec = nullptr;
-  // a first un-captured step of the stage path sets its kernels' attributes
+  RecordedGraph graph;
+  // a first step of the stage path, launched directly, sets its kernels' attributes
   for (auto& G : B.groups) DWF_TRY(g_cg_step(*G, B.st));
+  auto persistent = [](const Group& G) { return G.post_struct && G.sgather >= 0; };
+  auto decided_chunk = [&](Group& G) -> dwf_status {
+    return persistent(G) ? launch_chunk(G, G.sgather, G.sgrid) : stage_chunk(G);
+  };
   // Groups share nothing, so where all of them run as stage launches each is a branch of the
   // graph of its own: a group of a few tiles (a fraction of a wave per launch) runs beside a
   // large one instead of after it (12 problems, 384 + 1616 + 64 tiles: 235 ms against 270 one
   // after another).  Persistent launches stay alone on the GPU.
-  auto fork_join = [&]() -> dwf_status {
-    cudaEvent_t ev[2] = {};
-    for (auto& e : ev) DWF_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-    auto all = [&]() -> dwf_status {
-      DWF_CUDA(cudaEventRecord(ev[0], B.st));
-      for (size_t gi = 1; gi < B.groups.size(); gi++) {
-        cudaStream_t q = B.side[gi - 1];
-        DWF_CUDA(cudaStreamWaitEvent(q, ev[0], 0));
-        DWF_TRY(stage_chunk(*B.groups[gi], q));
-      }
-      DWF_TRY(stage_chunk(*B.groups[0], B.st));
-      for (size_t gi = 1; gi < B.groups.size(); gi++) {
-        DWF_CUDA(cudaEventRecord(ev[1], B.side[gi - 1]));
-        DWF_CUDA(cudaStreamWaitEvent(B.st, ev[1], 0));
+  auto record = [&]() {
+    bool branches = true;
+    for (auto& G : B.groups) branches = branches && !persistent(*G);
+    graph.record([&](GraphRecorder& rec) -> dwf_status {
+      for (auto& G : B.groups) {
+        if (branches) rec.last = nullptr;
+        DWF_TRY(decided_chunk(*G));
       }
       return DWF_OK;
-    };
-    const dwf_status s = all();
-    for (auto& e : ev) cudaEventDestroy(e);
-    return s;
+    });
   };
-  auto capture = [&]() -> dwf_status {
-    bool branches = B.groups.size() > 1;
-    for (auto& G : B.groups) branches = branches && !(G->post_struct && G->sgather >= 0);
-    while (branches && B.side.size() + 1 < B.groups.size()) {
-      cudaStream_t q;
-      DWF_CUDA(cudaStreamCreateWithFlags(&q, cudaStreamNonBlocking));
-      B.side.push_back(q);
-    }
-    DWF_CUDA(cudaStreamSynchronize(B.st));
-    DWF_CUDA(cudaStreamBeginCapture(B.st, cudaStreamCaptureModeThreadLocal));
-    dwf_status s = DWF_OK;
-    if (branches) {
-      s = fork_join();
-    } else {
-      for (auto& Gp : B.groups) {
-        Group& G = *Gp;
-        if (s == DWF_OK)
-          s = (G.post_struct && G.sgather >= 0) ? launch_chunk(G, G.sgather, G.sgrid)
-                                                : stage_chunk(G, B.st);
-      }
-    }
-    if (s != DWF_OK) {
-      cudaStreamEndCapture(B.st, &graph);
-      cudaGetLastError();
-      if (graph) cudaGraphDestroy(graph);
-      graph = nullptr;
-      return s;
-    }
-    DWF_CUDA(cudaStreamEndCapture(B.st, &graph));
-    DWF_CUDA(cudaGraphInstantiate(&exec, graph, 0));
-    return DWF_OK;
-  };
-  if (ntune == 0) DWF_TRY(capture());
+  if (ntune == 0) record();
   // one chunk of every group: a tuning round (timed launches of the next candidate) or the
-  // captured graph
+  // recorded graph
   auto run_chunk = [&]() -> dwf_status {
     if (tune_round >= ntune) {
-      DWF_CUDA(cudaGraphLaunch(exec, B.st));
+      if (graph.exec) DWF_CUDA(cudaGraphLaunch(graph.exec, B.st));
+      else for (auto& G : B.groups) DWF_TRY(decided_chunk(*G));
       return DWF_OK;
     }
     for (size_t gi = 0; gi < B.groups.size(); gi++) {
       Group& G = *B.groups[gi];
       if (!G.post_struct || cands[gi].empty()) {   // stage launches only, or decided earlier
-        if (G.post_struct && G.sgather >= 0) DWF_TRY(launch_chunk(G, G.sgather, G.sgrid));
-        else DWF_TRY(stage_chunk(G, B.st));
+        DWF_TRY(decided_chunk(G));
         continue;
       }
       const Cand& c = cands[gi][std::min(tune_round, cands[gi].size() - 1)];
       DWF_CUDA(cudaEventRecord(tev[0], B.st));
-      if (c.gather < 0) DWF_TRY(stage_chunk(G, B.st));
+      if (c.gather < 0) DWF_TRY(stage_chunk(G));
       else DWF_TRY(launch_chunk(G, c.gather, c.grid));
       DWF_CUDA(cudaEventRecord(tev[1], B.st));
       DWF_CUDA(cudaEventSynchronize(tev[1]));
@@ -1012,7 +970,7 @@ extern "C" dwf_status dwf_batch_solve(int n, const dwf_problem* problems, double
           fprintf(stderr, "\n");
         }
       }
-      DWF_TRY(capture());
+      record();
     }
     return DWF_OK;
   };
@@ -1081,8 +1039,6 @@ extern "C" dwf_status dwf_batch_solve(int n, const dwf_problem* problems, double
     (void)any_ru;
     if (all_done) break;
   }
-  if (exec) cudaGraphExecDestroy(exec);
-  if (graph) cudaGraphDestroy(graph);
   cudaEventDestroy(tev[0]);
   cudaEventDestroy(tev[1]);
   for (auto& Gp : B.groups) {   // a bounded device wait that gave up invalidates the solve

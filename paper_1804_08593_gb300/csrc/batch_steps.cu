@@ -90,18 +90,7 @@ static cudaError_t batch_launch_lg(const BatchStepArgs& b, int grid, int* cap, i
     *cap = per_sm * nsm;
     return cudaSuccess;
   }
-  // a cooperative launch through the extensible API (capturable in a CUDA graph)
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(32, LS);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k, b);
+  return launch_kernel(LAUNCH_COOPERATIVE, k, dim3((unsigned)grid), dim3(32, LS), smem, st, b);
 }
 
 template <int LS>

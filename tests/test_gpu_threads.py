@@ -104,3 +104,28 @@ def test_mspcg_beside_another_thread(flexible, other, blocking):
     assert all(np.array_equal(g, alone) for g in got)
     h.close()
     free()
+
+
+@pytest.mark.parametrize("form", ["stages", "persistent"])
+def test_batch_beside_another_thread(form, monkeypatch):
+    import torch
+    dwf = lib()
+    monkeypatch.setenv("DWF_BATCH_FORM", form)
+    rng = np.random.default_rng(41)
+    probs = []
+    for dims, Ls, mf in (((4, 4, 4, 4), 4, 0.1), ((4, 4, 4, 8), 8, 0.05), ((4, 6, 2, 6), 8, 0.2)):
+        phi = cuda(inputs.even_source(dims, Ls, rng))
+        probs.append(dict(dims=dims, Ls=Ls, M5=1.8, mf=mf, b=1.5, c=0.5, phi=phi,
+                          links=cuda(inputs.gauge_links(dims, 0.3, rng)), x=torch.zeros_like(phi)))
+    torch.cuda.synchronize()
+
+    def solve():
+        st = dwf.dwf_batch_solve(probs, 1e-10, 20000)
+        assert all(s["true_residual"] <= 1e-10 for s in st)
+        return [host(p["x"]) for p in probs]
+
+    solve()                # the chunk's launch shape is decided
+    alone = solve()
+    got, errors = _beside("device_wait", solve, 8)
+    assert not errors, errors
+    assert all(np.array_equal(a, b) for g in got for a, b in zip(g, alone))
