@@ -19,7 +19,9 @@ LIB = os.path.join(HERE, "lib", "libdwf.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 STAGE_PRECS = (0, 1, 2, 3)          # FP64, FP32, FP16, BF16
 STAGE_LS = (4, 6, 8, 10, 12, 16)    # fifth-dimension extents with compiled stage kernels
-FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
+# no -lineinfo: line tables are two thirds of a build (291 MB of objects and a 288 MB library with
+# them, 99 and 97 without); pass it as `extra` to see source lines in a profiler
+FLAGS = ["-O3", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
          "--expt-relaxed-constexpr", "-I", INCLUDE, "-I", CSRC]
 
 
