@@ -27,6 +27,9 @@ static cudaError_t launch_stage_p(const StageArgs& a, int Ls, bool dag, bool blo
 
 cudaError_t launch_stage_prec(int prec, const StageArgs& args, int Ls, bool dag, bool blocked,
                               cudaStream_t st) {
+  // the FP32 and 16-bit kernels take the local term's dagger from the stage's
+  if (args.local_mode != LOC_NONE && (args.local_mode == LOC_M5DAG) != dag)
+    return cudaErrorInvalidValue;
   StageArgs a = args;
   finish_stage_args(a, Ls, dag);
   switch (prec) {
