@@ -77,14 +77,6 @@ struct StageArgs {
   int grid;              // CTAs of a persistent launch (0: one CTA per tile)
 };
 
-template <typename A>
-__device__ __forceinline__ Coef5<A> coef5(const StageArgs& a) {
-  if constexpr (sizeof(A) == 8) return a.k64; else return a.k32;
-}
-template <typename A>
-__device__ __forceinline__ Coef5<A> coef5(const BatchSeg& S) {
-  if constexpr (sizeof(A) == 8) return S.k64; else return S.k32;
-}
 inline void finish_stage_args(StageArgs& a, int Ls, bool dag) {
   a.hs32 = (float)a.hop_scale;
   const double pre = a.post_pre != 0.0 ? a.post_pre : 1.0;
@@ -702,7 +694,7 @@ __device__ __forceinline__ bool stage_tile(const StageArgs& a, long tile,
   }
   const bool valid = jl < vh;
   // this tile's fifth-dimension coefficients (per problem when batched), read where used
-  auto K5 = [&]() -> Coef5<A> { return a.tile_seg ? coef5<A>(a.segp[seg]) : coef5<A>(a); };
+  auto K5 = [&]() -> Coef5<float> { return a.tile_seg ? a.segp[seg].k32 : a.k32; };
 
   Spinor<A> acc[NSL];
 #pragma unroll
@@ -934,8 +926,7 @@ __device__ __forceinline__ bool stage_tile(const StageArgs& a, long tile,
   for (int jj = 0; jj < NSL; jj++) {
     const int s = w + jj * LSP;
     Spinor<A>& acc_j = acc[jj];
-    A hs;
-    if constexpr (sizeof(A) == 8) hs = a.hop_scale; else hs = a.hs32;
+    const A hs = a.hs32;
   #pragma unroll
     for (int k = 0; k < 12; k++) acc_j.c[k] = cscale(hs, acc_j.c[k]);
 

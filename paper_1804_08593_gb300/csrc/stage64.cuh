@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(stage64_threads(DS), DS == 1 ? 2 : 1)
   }
   double nrm = 0.0;
   if (!owner) {
-    // its share belongs to the first four groups
+    // the first twelve groups hold the components
   } else if (a.epi == EPI_CG_R) {
     const double al = a.alpha[seg];
     double2* r = reinterpret_cast<double2*>(a.r) + site;

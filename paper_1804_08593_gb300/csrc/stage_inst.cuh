@@ -230,11 +230,9 @@ static cudaError_t stage_launch_one(const StageArgs& a, cudaStream_t st) {
 template <int LS, bool DAG, bool BLK, int POST, int DS>
 static cudaError_t stage64_launch(const StageArgs& a, int lst, cudaStream_t st) {
   auto k = stage64_kernel<LS, DAG, BLK, POST, DS>;
+  // every shape fits what a kernel gets without asking (48 KB, static shared memory included)
+  static_assert(8 * (stage64_hop_doubles(DS) * stage64_threads(DS) / DS + 2 * LS * LS) <= 47 * 1024);
   const size_t sm = stage64_smem(LS, POST, 1 << lst, DS);
-  if (sm > 40 * 1024) {   // 48 KB without asking, static shared memory included
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-  }
   const long ctas = a.ntiles * 32 >> lst;
   return launch_kernel(ctas <= sm_count() ? LAUNCH_EARLY : LAUNCH_PLAIN, k, dim3((unsigned)ctas),
                        dim3((unsigned)((LS << lst) * DS)), sm, st, a, lst);
