@@ -20,14 +20,8 @@ cudaError_t GraphRecorder::kernel(const void* k, dim3 grid, dim3 block, size_t s
   p.kernel.blockDim = block;
   p.kernel.sharedMemBytes = (unsigned)smem;
   p.kernel.kernelParams = args;   // copied by the call
-  cudaGraphEdgeData e{};
-  if (m == LAUNCH_EARLY) {
-    e.type = cudaGraphDependencyTypeProgrammatic;
-    e.from_port = cudaGraphKernelNodePortProgrammatic;
-  }
   cudaGraphNode_t n = nullptr;
-  cudaError_t r = cudaGraphAddNode(&n, graph, last ? &last : nullptr, last ? &e : nullptr,
-                                   last ? 1 : 0, &p);
+  cudaError_t r = cudaGraphAddNode(&n, graph, last ? &last : nullptr, nullptr, last ? 1 : 0, &p);
   if (r == cudaSuccess && m == LAUNCH_COOPERATIVE) {
     cudaLaunchAttributeValue v{};
     v.cooperative = 1;

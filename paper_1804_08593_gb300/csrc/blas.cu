@@ -38,7 +38,7 @@ static cudaError_t vec_launch(const VecArgs& a, cudaStream_t st) {
   static std::atomic<uint64_t> attr{0};
   cudaError_t e = set_smem_once(vec_kernel<P, LS>, attr, (int)(LS * 24 * 32 * sizeof(A)));
   if (e != cudaSuccess) return e;
-  const bool early = P == P64 && a.Vp / w <= sm_count();
+  const bool early = P == P64 && early_launch(a.Vp / w, a.stop);
   return launch_kernel(early ? LAUNCH_EARLY : LAUNCH_PLAIN, vec_kernel<P, LS>,
                        dim3((unsigned)(a.Vp / w)), dim3(w, LS), sm, st, a);
 }

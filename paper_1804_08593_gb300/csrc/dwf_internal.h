@@ -284,12 +284,17 @@ struct RecordedGraph {
 // Clears device memory in stream order, or records that.
 cudaError_t clear_async(void* p, size_t bytes, cudaStream_t st);
 
-// Launches a kernel, or records that.  LAUNCH_EARLY, for kernels that begin with
-// programmatic_start(): the CTAs are already placed when the kernel in front of it on the stream
-// ends.  For grids of at most one CTA per SM
-// only (FP64 solvers on the smallest lattices are chains of 10 us kernels: CG on 4^4 x 8 20.3 ->
-// 18.9 ms); a larger grid is placed wherever the running one happens to leave room, which
-// undoes the even spread that the FP64 stages depend on (8^3x16 x 8: 59 us a stage became 90).
+// Whether an FP64 kernel of this many CTAs is launched early (LAUNCH_EARLY): its CTAs are placed
+// before the kernel in front of it on the stream ends, which hides the launches of a single
+// application (4^4 x 8, Moebius: 65.2 -> 53.8 us a call).  Not in a solver's iterations, whose
+// launches carry a stop flag (4^4 x 8: 16 iterations launched one by one took 1.21 ms with it,
+// 1.10 without; replayed from a graph 59 and 42 us an iteration), and for at most one CTA per SM:
+// a larger grid is placed wherever the running one leaves room, which undoes the even spread that
+// these kernels depend on (8^3x16 x 8: 260 us an iteration became 426).
+inline bool early_launch(long ctas, const int* stop) { return !stop && ctas <= sm_count(); }
+
+// Launches a kernel, or records that (LAUNCH_EARLY, for kernels that begin with
+// programmatic_start(), as a plain one).
 template <typename... A>
 cudaError_t launch_kernel(LaunchMode m, void (*k)(A...), dim3 grid, dim3 block, size_t smem,
                           cudaStream_t st, A... args) {

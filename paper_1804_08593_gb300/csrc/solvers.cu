@@ -217,13 +217,13 @@ static dwf_status cg_iteration(const OpEngine& E, const CGVectors& v, double* ds
 }
 
 // Eight CG iterations as a CUDA graph, replayed through the solve, for lattices whose kernels
-// are shorter than the host takes to launch them (4^4 x 8, Shamir: 58 us an iteration launched one
-// by one, 45 replayed).  Every iteration of a solve has the same arguments, but for the place in
-// the caller's history after a restart (`same` false: launched directly).  Recording takes the
-// host about 150 us, which the second replay has earned back (24 iterations in all, f64 4^4 x 8:
-// 1.75 ms with a graph, 1.76 without; one replay only, 16 iterations: 1.30 and 1.15; 40: 2.69 and
-// 2.84; 120: 7.25 and 8.95): it waits for a chunk of two.  Not while the profiler records events
-// per launch or inside a caller's capture.
+// are shorter than the host takes to launch them (FP64 4^4 x 8, Shamir: 51 us an iteration
+// launched one by one, 40 replayed).  Every iteration of a solve has the same arguments, but for
+// the place in the caller's history after a restart (`same` false: launched directly).  Recording
+// costs the host 30 to 50 us more than launching the same iterations; it waits for a chunk of two
+// replays, from which on no length of solve loses by it (8 iterations in all: 0.65 ms if
+// recorded, 0.61 if launched; 24: 1.39 and 1.45; 120: 5.26 and 6.39).  Not while the profiler
+// records events per launch or inside a caller's capture.
 struct CgGraph {
   static constexpr int N = 8;
   static constexpr long MOST = 200000;   // sites x slices of one parity

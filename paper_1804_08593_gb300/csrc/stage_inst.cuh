@@ -234,8 +234,8 @@ static cudaError_t stage64_launch(const StageArgs& a, int lst, cudaStream_t st) 
   static_assert(8 * (stage64_hop_doubles(DS) * stage64_threads(DS) / DS + 2 * LS * LS) <= 47 * 1024);
   const size_t sm = stage64_smem(LS, POST, 1 << lst, DS);
   const long ctas = a.ntiles * 32 >> lst;
-  return launch_kernel(ctas <= sm_count() ? LAUNCH_EARLY : LAUNCH_PLAIN, k, dim3((unsigned)ctas),
-                       dim3((unsigned)((LS << lst) * DS)), sm, st, a, lst);
+  return launch_kernel(early_launch(ctas, a.stop) ? LAUNCH_EARLY : LAUNCH_PLAIN, k,
+                       dim3((unsigned)ctas), dim3((unsigned)((LS << lst) * DS)), sm, st, a, lst);
 }
 template <int LS, bool DAG, bool BLK, int POST>
 static cudaError_t stage64_launch_ds(const StageArgs& a, cudaStream_t st) {
