@@ -436,7 +436,7 @@ __device__ void grid_reduce_seg(const RedArgs& r, T (&v)[NV], double* scratch, l
     for (int i = 0; i < NV; i++) s[i] = 0.0;
     // FP64 stages have small CTAs and up to one partial per site: several loads in flight per
     // thread, added in the same order as one by one (this CTA's L2 latency is the tail of the
-    // whole launch; 8^3x16 x 8: 1.3 us of 69)
+    // whole launch; 8^3x16 x 8, the adjoint stage with the residual update: 69.1 -> 67.8 us)
     constexpr int U = sizeof(T) == 8 ? 8 : 1;
     for (int k = tid; k < ntiles; k += U * nthr) {
       double x[U][NV];

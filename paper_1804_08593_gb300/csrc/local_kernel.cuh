@@ -684,7 +684,7 @@ __device__ __forceinline__ void write_partial(A v, A (*red)[32], double* dst, in
 // share in order, four loads in flight, then warp 0 the shares (a fixed order for a given C).
 // An FP64 addition takes 64 cycles of an SM quarter: one warp adding all 304 partials of a slot
 // that has the whole GPU took 10 us, twice an iteration (12^3x24, 32 blocks of 6^4, Ls = 12,
-// l = 6: 1.42 -> 1.22 ms a launch; 8^3x16, 4^4 blocks, Ls = 4: 0.66 -> 0.41 ms).
+// l = 6: 1.40 -> 1.22 ms a launch; 8^3x16, 4^4 blocks, Ls = 4: 0.66 -> 0.41 ms).
 template <int NW>
 __device__ __forceinline__ double slot_total(const double* part, int C, double (*sc)[32], int w,
                                              int lane) {

@@ -17,9 +17,10 @@
 //    groups of threads (direction and half-spinor component) on lattices too small to fill
 //    the chip with whole hops; lst and DS are chosen at launch (stage64_shape).
 //
-// Measured, us per launch (stage A; before: one CTA per 32 sites, every instruction above):
-// 4^4 x 8 65 -> 8, 8^3x16 x 8 73 -> 56, 12^4 x 12 282 -> 212, 16^4 x 16 1019 -> 850 (94 % of the
-// FP64 rate on the instructions left), 16^3x32 x 12 1499 -> 1275.
+// Measured, us per launch of the stage with the recurrence post (before: one CTA per 32 sites,
+// every instruction above): 4^4 x 8 74 -> 7, 8^3x16 x 8 74 -> 59, 12^4 x 12 325 -> 224,
+// 16^4 x 16 1020 -> 870 (92 % of the FP64 rate on the instructions left), 16^3x32 x 12
+// 1498 -> 1298.
 #pragma once
 
 #include "stage.cuh"
@@ -134,7 +135,7 @@ inline size_t stage64_smem(int Ls, int post, int st, int ds) {
 }
 
 // Whole hops: two CTAs' worth of registers (168 a thread) keep three warps per SM quarter
-// resident (12^4 x 12: 974 us a CG iteration; with the 186 that the compiler takes freely 1034).
+// resident (12^4 x 12: 964 us a CG iteration; with the 186 that the compiler takes freely 1028).
 template <int LS, bool DAG, bool BLOCKED, int POST, int DS>
 __global__ void __launch_bounds__(stage64_threads(DS), DS == 1 ? 2 : 1)
     stage64_kernel(const StageArgs a, const int lst) {
@@ -430,9 +431,10 @@ __global__ void __launch_bounds__(stage64_threads(DS), DS == 1 ? 2 : 1)
 // least FP64 work: a quarter takes 64 cycles per warp-wide FP64 instruction, so its work is
 // its warps times their FP64 instructions, about 1000 with whole hops and 110 with a direction
 // and half-spinor component per thread.  Among equals the smaller CTA, whose warps spread more
-// evenly, unless a load would fetch less than 64 contiguous bytes.  Measured per stage launch:
-// 16^4 x 16, whole hops, 2 / 4 / 8 / 16 sites: 844 / 816 / 810 / 924 us; 8^3x16 x 8, 4 / 8 / 32
-// sites: 55 / 63 / 64 us.
+// evenly, unless a load would fetch less than 64 contiguous bytes.  Measured per launch of the
+// stage with the recurrence post, whole hops: 16^4 x 16, 2 / 4 (chosen) / 8 sites: 898 / 870 /
+// 866 us; 12^4 x 12, 8 (chosen) / 16: 224 / 243; 8^3x16 x 8, 4 (chosen) / 8 / 16: 59 / 67 / 67, with
+// direction groups 70 to 73.
 struct Stage64Shape {
   int lst, ds;
 };

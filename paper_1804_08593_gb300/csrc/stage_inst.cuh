@@ -102,13 +102,15 @@ static void stage_cands(StageCand* c, int& n) {
 }
 
 // FP32: which of the three variants above runs, by size (no timing: a solver's launches carry a
-// stop flag and are never timed).  The L2-to-SM traffic of the neighbour spinors bounds them
-// (about 8 TB/s: neither half the instructions nor twice the loads in flight changes the large
-// sizes by 5 %), so the packed component form wins by its registers, except where a CTA of Ls
-// warps leaves a second one no room: Ls = 16 pairs the slices (16^4: 240 us for the four stages
-// of a CG step against 297; at Ls = 12 it is level within 3 % on one problem and 7 % behind in
-// batches).  Up to two tiles per SM the links' L2 prefetch only delays the loads (8^3x16 x 12:
-// 37.2 us for the four stages against 38.6; 12^4 x 12: 85.3 both).
+// stop flag and are never timed).  What bounds them is the latency of the neighbour spinors, half
+// of which come from L2 (24^4 x 12, recurrence post: 7.2 TB/s from L2, 2.6 from DRAM, 42 % of the
+// issue slots, 6.5 warps waiting for a load per instruction issued, all 24 resident warps in
+// flight; half the instructions or twice the loads in flight change the large sizes by less than
+// 5 %).  So the packed component form wins by its registers, except where a CTA of Ls warps leaves
+// a second one no room: Ls = 16 pairs the slices (16^4: 247 us for the four stages of a CG step
+// against 289; at Ls = 12 it is 9 % behind, 24^3x48: 1 759 us against 1 620).  Up to two tiles
+// per SM the links' L2 prefetch only delays the loads (8^3x16 x 12: 36.0 us for the four stages
+// against 37.7; 12^4 x 12: 84 both).
 template <int LS>
 static int stage_rule32(long ntiles) {
   if (LS == 16) return 1;
