@@ -220,15 +220,16 @@ static dwf_status cg_iteration(const OpEngine& E, const CGVectors& v, double* ds
 // are shorter than the host takes to launch them (FP64 4^4 x 8, Shamir: 51 us an iteration
 // launched one by one, 40 replayed).  Every iteration of a solve has the same arguments, but for
 // the place in the caller's history after a restart (`same` false: launched directly).  Recording
-// costs the host 30 to 50 us more than launching the same iterations; it waits for a chunk of two
-// replays, from which on no length of solve loses by it (8 iterations in all: 0.65 ms if
-// recorded, 0.61 if launched; 24: 1.39 and 1.45; 120: 5.26 and 6.39).  Not while the profiler
-// records events per launch or inside a caller's capture.
+// costs the host 30 to 50 us more than launching the same iterations: not for the first chunk of a
+// solve, and only where the limit on the iterations leaves room for two replays, from which on no
+// length of solve loses by it (8 iterations in all: 0.65 ms if recorded, 0.61 if launched; 24:
+// 1.39 and 1.45; 120: 5.26 and 6.39).  Not while the profiler records events per launch or inside
+// a caller's capture.
 struct CgGraph {
   static constexpr int N = 8;
   static constexpr long MOST = 200000;   // sites x slices of one parity
   RecordedGraph graph;
-  bool usable;
+  bool usable, warm = false;
   explicit CgGraph(const OpEngine& E) {
     const dwf_ctx* h = E.h;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -237,14 +238,15 @@ struct CgGraph {
              cs == cudaStreamCaptureStatusNone;
   }
   template <typename F>
-  dwf_status iterations(dwf_ctx* h, int n, bool same, F one) {
-    if (usable && same && n >= 2 * N) {
+  dwf_status iterations(dwf_ctx* h, int n, int left, bool same, F one) {
+    if (usable && same && warm && n >= N && left >= 2 * N) {
       usable = false;   // once
       graph.record([&](GraphRecorder&) -> dwf_status {
         for (int k = 0; k < N; k++) DWF_TRY(one());
         return DWF_OK;
       });
     }
+    warm = true;
     for (; graph.exec && same && n >= N; n -= N) DWF_CUDA(cudaGraphLaunch(graph.exec, h->stream));
     for (; n > 0; n--) DWF_TRY(one());
     return DWF_OK;
@@ -356,9 +358,9 @@ static dwf_status run_cg(dwf_ctx* h, Layout* lay, const void* b_c128, void* x_c1
     int fl[F_NFLAG] = {0};
     bool finite_cycle = true;
     while (true) {
-      const int n = std::min(chunk, maxit - iters - done_cycle);
+      const int left = maxit - iters - done_cycle, n = std::min(chunk, left);
       if (n <= 0) break;
-      DWF_TRY(graph.iterations(h, n, !dhist || total_hist == 0, [&]() {
+      DWF_TRY(graph.iterations(h, n, left, !dhist || total_hist == 0, [&]() {
         return cg_iteration(E, v, dsc, dfl, dhist ? dhist + total_hist : nullptr,
                             dcurv ? dcurv + total_hist : nullptr, dhist ? hcap - total_hist : 0);
       }));

@@ -17,7 +17,8 @@ def _problem(dims, Ls, b, c):
 
 @pytest.mark.parametrize("maxit,replayed", [(16, False), (23, False), (24, True), (56, True)])
 def test_short_solves_record_no_graph(maxit, replayed):
-    """Chunks of 8, 16, 32 iterations: a graph of 8 is recorded in a chunk of at least 16."""
+    """Chunks of 8, 16, 32 iterations: a graph of 8 is recorded after the first chunk, if at least
+    16 more may follow."""
     import torch
     from torch.profiler import ProfilerActivity, profile
     dwf = lib()
